@@ -161,6 +161,23 @@ inline void ff_split(double d, float* hi, float* lo) {
     *lo = (float)(d - (double)*hi);
 }
 
+// n / d as (n * m) >> k, exact for 0 <= n < 2^24 and 1 <= d < 2^12
+// (m = ceil(2^k / d) with k = 24 + ceil(log2 d): the round-up reciprocal of
+// Granlund and Montgomery, which fits 32 bits here).
+struct FastDiv {
+    uint32_t m;
+    int k;
+};
+inline FastDiv make_fastdiv(uint32_t d) {
+    int s = 0;
+    while ((1u << s) < d) ++s;
+    const int k = 24 + s;
+    return FastDiv{(uint32_t)(((1ull << k) + d - 1) / d), k};
+}
+__device__ __forceinline__ int fdiv(int n, const FastDiv& f) {
+    return (int)(((uint64_t)(uint32_t)n * f.m) >> f.k);
+}
+
 constexpr double LOG_2PI = 1.8378770664093454835606594728112;
 
 // Periodic neighbour wrap for |offset| <= L.

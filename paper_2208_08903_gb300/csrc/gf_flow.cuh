@@ -20,6 +20,7 @@ namespace gf {
 //                                          <- h2 of slices s0-1 .. s0+n in in[0..n+2)
 constexpr int PH_H1 = 0, PH_H2 = 1, PH_C3 = 2;
 constexpr int MAX_PHASE_SLICES = 62;
+constexpr int kF32Tiles = 7, kCtaSizes = 4;   // fused FP32 kernel: conv2 tiles; CTAs of 64 << i threads
 
 struct Phase {
     uint8_t type, n;
@@ -51,7 +52,13 @@ struct gf_flow {
     int R;                  // slots per hidden tensor
     bool full;
     size_t smem_bytes;
-    bool wsmem;             // FP32 kernel keeps all packed weights in shared memory
+    // fused FP32 kernel (gf_flow_fp32.cu): staged taps of W2 per buffer, a
+    // second buffer for the other weights, or weights read from global memory;
+    // lanes per site of the head's sums; conv2 phases of a layer by slice count
+    int stage_taps;
+    bool two_small, weights_global;
+    int head_G, head_zb, head_a, head_b;
+    int16_t h2_count[gf::MAX_PHASE_SLICES + 1];
     // BF16 tensor-core path: the 3D L=16, C=32 kernel (gf_flow_bf16.cu) or,
     // when tc is set, the kernel for other shapes (gf_flow_tc.cu)
     void* d_bf16;           // per-layer weight blocks of the tensor-core kernel
@@ -89,8 +96,9 @@ gf_status repack_weights(gf_flow* f, cudaStream_t stream);  // d_canon -> d_pack
 gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, int64_t B,
                            uint64_t seed, uint64_t counter0, const float* z_in, float* z_out,
                            const float* phi_in, float* phi_out, double* logq_out,
-                           double* S_out, double* logw_out, cudaStream_t stream);
-gf_status flow_fp32_configure(gf_flow* f);   // chooses FULL/RING, G, smem
+                           double* S_out, double* logw_out, cudaStream_t stream, float* xs_out = nullptr,
+                           int64_t xs_stride = 0, double* logdet_out = nullptr);
+gf_status flow_fp32_configure(gf_flow* f);   // chooses FULL/RING, G, staging, smem
 
 // 3D L=16, hidden 32, FP32 (gf_flow_fp32_c32.cu)
 bool fp32_c32_supported(const gf_flow* f);

@@ -1,0 +1,11 @@
+// gf_flow_fp32_2d_w24.cu -- the 2D, width 24 instantiations of the fused FP32 kernel.
+#include "gf_flow_fp32_kernel.cuh"
+
+namespace gf {
+namespace f32k {
+
+template <>
+FlowKernel kernel_of<2, 24>(int tile, bool gw) { return pick_kernel<2, 24>(tile, gw); }
+
+}  // namespace f32k
+}  // namespace gf

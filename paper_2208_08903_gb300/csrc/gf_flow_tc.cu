@@ -82,23 +82,6 @@ constexpr int kTcMaxTiles = 64;           // tiles per layer (one completion bar
 constexpr long long kTcWaitLimit = 1ll << 22;
 constexpr int kSmemPerCTA = 232448;       // 227 KB opt-in maximum per CTA
 
-// n / d as (n * m) >> k, exact for 0 <= n < 2^24 and 1 <= d < 2^12
-// (m = ceil(2^k / d) with k = 24 + ceil(log2 d): the round-up reciprocal of
-// Granlund and Montgomery, which fits 32 bits here).
-struct FastDiv {
-    uint32_t m;
-    int k;
-};
-FastDiv make_fastdiv(uint32_t d) {
-    int s = 0;
-    while ((1u << s) < d) ++s;
-    const int k = 24 + s;
-    return FastDiv{(uint32_t)(((1ull << k) + d - 1) / d), k};
-}
-__device__ __forceinline__ int fdiv(int n, const FastDiv& f) {
-    return (int)(((uint64_t)(uint32_t)n * f.m) >> f.k);
-}
-
 struct TcGeom {
     int nd, L, V, P, C, Cp, T;
     int p_first;          // padded position of site (0, ..., 0) = 1 + P (+ P^2); also the largest tap offset
