@@ -13,18 +13,22 @@
 //    memory directly (a warp per configuration or a block per configuration).
 //  - chain gather: the chain's series O[chain_idx[k]] of a per-proposal
 //    observable.
-//  - Gamma(t) of a series (one CTA per lag, fixed-order FP64 reduction), then
-//    the Madras-Sokal automatic window for tau_int in one thread.
+//  - Gamma(t) of a series (a CTA takes up to eight lags, fixed-order FP64
+//    reduction), then the Madras-Sokal automatic window for tau_int in one warp.
 //  - ESS fraction (sum w)^2 / (n sum w^2) of w = exp(log w), the largest
-//    log w factored out.
+//    log w factored out (one cluster of CTAs).
 #include <algorithm>
 #include <cmath>
+
+#include <cooperative_groups.h>
 
 #include "gf_async.cuh"
 #include "gf_common.cuh"
 
 namespace gf {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kObsThreads = 256;
 constexpr int kRedThreads = 1024;
@@ -294,91 +298,187 @@ __global__ void gather_kernel(int64_t n, const int64_t* __restrict__ chain_idx, 
     }
 }
 
-// dbar = mean of (y_k - y_0), one block, fixed order.  Stored in out[3].
-__global__ void __launch_bounds__(kRedThreads) mean_dev_kernel(int64_t n, const double* __restrict__ y,
-                                                              double* __restrict__ out) {
-    __shared__ double red[32];
-    const double y0 = y[0];
-    double acc = 0.0;
-    for (int64_t k = threadIdx.x; k < n; k += blockDim.x) acc += y[k] - y0;
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) out[3] = acc / (double)n;
-}
+// The reductions over a series run as one cluster of kRedCluster CTAs (one for
+// short series): FP64 instructions take about 19 cycles of an SM per warp, so a
+// single CTA is bound by its SM's FP64 pipe, and a cluster combines its CTAs'
+// sums through distributed shared memory without scratch memory or a second
+// launch.  Fixed order: rank by rank.  Measured on 16,384 values against one CTA:
+// ESS 112 -> 32 us, mean 24 -> 10 us.
+constexpr int kRedCluster = 8;
+constexpr int64_t kRedClusterMinN = 2048;
 
-// Gamma(t) for t = blockIdx.x (grid-stride over lags).
-__global__ void __launch_bounds__(kObsThreads) gamma_kernel(int64_t n, const double* __restrict__ y, int t_max,
-                                                           const double* __restrict__ stats,
-                                                           double* __restrict__ gamma) {
-    __shared__ double red[32];
-    const double y0 = y[0], dbar = stats[3];
-    for (int t = blockIdx.x; t <= t_max; t += gridDim.x) {
-        double acc = 0.0;
-        for (int64_t k = threadIdx.x; k + t < n; k += blockDim.x)
-            acc += ((y[k] - y0) - dbar) * ((y[k + t] - y0) - dbar);
-        acc = block_sum(acc, red);
-        if (threadIdx.x == 0) gamma[t] = acc / (double)(n - t);
-        __syncthreads();
+struct ClusterPos {
+    cg::cluster_group cl = cg::this_cluster();
+    int rank = (int)cl.block_rank(), size = (int)cl.num_blocks();
+    __device__ int64_t first() const { return (int64_t)rank * blockDim.x + threadIdx.x; }
+    __device__ int64_t stride() const { return (int64_t)size * blockDim.x; }
+    // v of every rank, combined by op in rank order (slot: a shared variable of this CTA)
+    template <typename Op>
+    __device__ double combine(double v, double* slot, Op op) {
+        if (threadIdx.x == 0) *slot = v;
+        cl.sync();
+        double r = *cl.map_shared_rank(slot, 0);
+        for (int i = 1; i < size; ++i) r = op(r, *cl.map_shared_rank(slot, i));
+        cl.sync();                                   // every rank has read it
+        return r;
     }
-}
-
-// Madras-Sokal window and the summary {tau, W, error, mean}; one thread.
-__global__ void window_kernel(int64_t n, const double* __restrict__ y, const double* __restrict__ gamma, int t_max,
-                              double c, double* __restrict__ out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const double mean = y[0] + out[3];
-    if (!(gamma[0] > 0.0)) {
-        out[0] = 0.5; out[1] = 0.0; out[2] = 0.0; out[3] = mean;
-        return;
-    }
-    double tau = 0.5;
-    int W = t_max;
-    for (int w = 1; w <= t_max; ++w) {
-        tau += gamma[w] / gamma[0];
-        if ((double)w >= c * tau) { W = w; break; }
-    }
-    out[0] = tau;
-    out[1] = (double)W;
-    out[2] = tau * sqrt((4.0 * W + 2.0) / (double)n);
-    out[3] = mean;
-}
+};
+__device__ __forceinline__ double dadd(double a, double b) { return a + b; }
+__device__ __forceinline__ double dmax(double a, double b) { return fmax(a, b); }
 
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
+// The block's N values combined per warp, then over the warps by thread 0..N-1
+// (valid in red_out[0 .. N) after the trailing barrier).
+template <int N, typename WarpOp, typename Op>
+__device__ void block_combine(const double (&v)[N], double (*red)[32], double* red_out, WarpOp wop, Op op) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const double w = wop(v[i]);
+        if (lane == 0) red[i][wid] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x < N) {
+        double r = red[threadIdx.x][0];
+        for (int w = 1; w < nw; ++w) r = op(r, red[threadIdx.x][w]);
+        red_out[threadIdx.x] = r;
+    }
+    __syncthreads();
+}
 
-// ESS fraction in one block: max, then sum w and sum w^2 in a fixed order.
+// dbar = mean of (y_k - y_0), one cluster, fixed order.  Stored in out[3].
+__global__ void __launch_bounds__(kRedThreads) mean_dev_kernel(int64_t n, const double* __restrict__ y,
+                                                              double* __restrict__ out) {
+    __shared__ double red[1][32], tot[1], slot;
+    ClusterPos c;
+    const double y0 = y[0];
+    double acc[1] = {0.0};
+    for (int64_t k = c.first(); k < n; k += c.stride()) acc[0] += y[k] - y0;
+    block_combine<1>(acc, red, tot, [](double v) { return warp_sum(v); }, dadd);
+    const double sum = c.combine(tot[0], &slot, dadd);
+    if (c.rank == 0 && threadIdx.x == 0) out[3] = sum / (double)n;
+}
+
+// Gamma(t) for LT consecutive lags per block (grid-stride): a tile of the
+// centred series is formed once in shared memory and read by every lag, so an
+// element costs 2 / LT subtractions and one multiply-add per lag instead of
+// four and one (16,384 values, 1,001 lags: 167 -> 70 us).  The FP64 pipe bounds it; LT = the lags divided by the SMs (at
+// most 8) keeps one block per SM.
+constexpr int kGammaTile = 1024, kGammaMaxLags = 8;
+template <int LT>
+__global__ void __launch_bounds__(kObsThreads) gamma_kernel(int64_t n, const double* __restrict__ y, int t_max,
+                                                           const double* __restrict__ stats,
+                                                           double* __restrict__ gamma) {
+    __shared__ double d[kGammaTile], e[kGammaTile + LT], red[LT][32], tot[LT];
+    const double y0 = y[0], dbar = stats[3];
+    const auto centred = [&](int64_t k) { return k < n ? (y[k] - y0) - dbar : 0.0; };
+    for (int t0 = blockIdx.x * LT; t0 <= t_max; t0 += gridDim.x * LT) {
+        double acc[LT];
+#pragma unroll
+        for (int l = 0; l < LT; ++l) acc[l] = 0.0;
+        for (int64_t k0 = 0; k0 + t0 < n; k0 += kGammaTile) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < kGammaTile; i += blockDim.x) d[i] = centred(k0 + i);
+            for (int i = threadIdx.x; i < kGammaTile + LT; i += blockDim.x) e[i] = centred(k0 + t0 + i);
+            __syncthreads();
+            // (the centred series is zero past its end: no bound per lag)
+            for (int i = threadIdx.x; i < kGammaTile; i += blockDim.x) {
+                const double v = d[i];
+#pragma unroll
+                for (int l = 0; l < LT; ++l) acc[l] = fma(v, e[i + l], acc[l]);
+            }
+        }
+        block_combine<LT>(acc, red, tot, [](double v) { return warp_sum(v); }, dadd);
+        if (threadIdx.x < LT && t0 + (int)threadIdx.x <= t_max)
+            gamma[t0 + threadIdx.x] = tot[threadIdx.x] / (double)(n - t0 - (int)threadIdx.x);
+    }
+}
+
+// Madras-Sokal window and the summary {tau, W, error, mean}; one warp: the
+// ratios of 32 lags at a time, added in order.
+__global__ void window_kernel(int64_t n, const double* __restrict__ y, const double* __restrict__ gamma, int t_max,
+                              double c, double* __restrict__ out) {
+    const int lane = threadIdx.x;
+    const double mean = y[0] + out[3], g0 = gamma[0];
+    double tau = 0.5;
+    int W = t_max;
+    if (g0 > 0.0) {
+        bool found = false;
+        for (int w0 = 1; w0 <= t_max && !found; w0 += 32) {
+            const double r = w0 + lane <= t_max ? gamma[w0 + lane] / g0 : 0.0;
+            for (int i = 0; i < 32 && w0 + i <= t_max; ++i) {
+                tau += __shfl_sync(0xffffffffu, r, i);
+                if ((double)(w0 + i) >= c * tau) { W = w0 + i; found = true; break; }
+            }
+        }
+    } else {
+        W = 0;
+    }
+    __syncwarp();
+    if (lane != 0) return;
+    out[0] = tau;
+    out[1] = (double)W;
+    out[2] = g0 > 0.0 ? tau * sqrt((4.0 * W + 2.0) / (double)n) : 0.0;
+    out[3] = mean;
+}
+
+// ESS fraction in one cluster: max, then sum w and sum w^2 in a fixed order.
 __global__ void __launch_bounds__(kRedThreads) ess_kernel(int64_t n, const double* __restrict__ logw,
                                                          double* __restrict__ out) {
-    __shared__ double red[32];
-    __shared__ double mx_s;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double mx = -INFINITY;
-    for (int64_t k = threadIdx.x; k < n; k += blockDim.x) mx = fmax(mx, logw[k]);
-    mx = warp_max(mx);
-    if (lane == 0) red[wid] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double m = -INFINITY;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmax(m, red[i]);
-        mx_s = m;
-    }
-    __syncthreads();
-    mx = mx_s;
-    if (!(mx > -INFINITY)) {                       // n == 0 or all weights zero
-        if (threadIdx.x == 0) *out = 0.0;
+    __shared__ double red[2][32], tot[2], slot;
+    ClusterPos c;
+    double mx[1] = {-INFINITY};
+    for (int64_t k = c.first(); k < n; k += c.stride()) mx[0] = fmax(mx[0], logw[k]);
+    block_combine<1>(mx, red, tot, [](double v) { return warp_max(v); }, dmax);
+    const double top = c.combine(tot[0], &slot, dmax);
+    if (!(top > -INFINITY)) {                      // n == 0 or all weights zero (the same in every rank)
+        if (c.rank == 0 && threadIdx.x == 0) *out = 0.0;
         return;
     }
-    double s1 = 0.0, s2 = 0.0;
-    for (int64_t k = threadIdx.x; k < n; k += blockDim.x) {
-        const double w = exp(logw[k] - mx);
-        s1 += w;
-        s2 += w * w;
+    double s[2] = {0.0, 0.0};
+    for (int64_t k = c.first(); k < n; k += c.stride()) {
+        const double w = exp(logw[k] - top);
+        s[0] += w;
+        s[1] += w * w;
     }
-    s1 = block_sum(s1, red);
-    s2 = block_sum(s2, red);
-    if (threadIdx.x == 0) *out = s1 * s1 / ((double)n * s2);
+    block_combine<2>(s, red, tot, [](double v) { return warp_sum(v); }, dadd);
+    const double s1 = c.combine(tot[0], &slot, dadd), s2 = c.combine(tot[1], &slot, dadd);
+    if (c.rank == 0 && threadIdx.x == 0) *out = s1 * s1 / ((double)n * s2);
+}
+
+// Launches a reduction over n elements as one cluster.
+template <typename... P, typename... A>
+bool launch_reduction(void (*kern)(P...), int64_t n, cudaStream_t stream, A... args) {
+    const unsigned size = n >= kRedClusterMinN ? kRedCluster : 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(kRedThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...) == cudaSuccess;
+}
+
+template <int LT = kGammaMaxLags>
+void launch_gamma(int lags_per_block, int64_t n, const double* y, int t_max, const double* stats, double* gamma,
+                  cudaStream_t stream) {
+    if constexpr (LT > 1) {
+        if (lags_per_block < LT) {
+            launch_gamma<LT - 1>(lags_per_block, n, y, t_max, stats, gamma, stream);
+            return;
+        }
+    }
+    const int64_t blocks = ((int64_t)t_max + LT) / LT;
+    gamma_kernel<LT><<<(unsigned)std::min<int64_t>(blocks, (int64_t)num_sms() * 8), kObsThreads, 0, stream>>>(
+        n, y, t_max, stats, gamma);
 }
 
 int64_t ipow(int64_t a, int e) {
@@ -434,10 +534,9 @@ gf_status gf_autocorr(int64_t n, const double* d_y, int32_t t_max, double c_wind
                       double* d_tau_out, cudaStream_t stream) {
     if (n < 1 || t_max < 0 || t_max >= n || !(c_window > 0.0)) return GF_EINVAL;
     if (!d_y || !d_gamma_out || !d_tau_out) return GF_EINVAL;
-    mean_dev_kernel<<<1, kRedThreads, 0, stream>>>(n, d_y, d_tau_out);
-    GF_CHECK_LAUNCH();
-    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)t_max + 1, (int64_t)num_sms() * 8);
-    gamma_kernel<<<grid, kObsThreads, 0, stream>>>(n, d_y, t_max, d_tau_out, d_gamma_out);
+    if (!launch_reduction(mean_dev_kernel, n, stream, n, d_y, d_tau_out)) return GF_ECUDA;
+    const int lags = (int)(((int64_t)t_max + num_sms()) / num_sms());
+    launch_gamma(std::min(lags, kGammaMaxLags), n, d_y, t_max, d_tau_out, d_gamma_out, stream);
     GF_CHECK_LAUNCH();
     window_kernel<<<1, 32, 0, stream>>>(n, d_y, d_gamma_out, t_max, c_window, d_tau_out);
     GF_CHECK_LAUNCH();
@@ -446,7 +545,7 @@ gf_status gf_autocorr(int64_t n, const double* d_y, int32_t t_max, double c_wind
 
 gf_status gf_ess(int64_t n, const double* d_logw, double* d_ess_out, cudaStream_t stream) {
     if (n < 0 || !d_ess_out || (n > 0 && !d_logw)) return GF_EINVAL;
-    ess_kernel<<<1, kRedThreads, 0, stream>>>(n, d_logw, d_ess_out);
+    if (!launch_reduction(ess_kernel, n, stream, n, d_logw, d_ess_out)) return GF_ECUDA;
     GF_CHECK_LAUNCH();
     return GF_OK;
 }
