@@ -119,8 +119,8 @@ __global__ void __launch_bounds__(kActThreads) action_kernel(int nd, int L, int 
 // sigma >= every term (M = max |phi| of the configuration, from a first pass
 // over the staged field): A and B only grow from sigma_A >= M^2 and
 // sigma_B >= M^4; H, whose terms have either sign, starts at
-// sigma_H >= (16 nd + 1) M^2 and is folded into a pair accumulator (and reset)
-// after every 2 x 4 sites, so its 8 nd terms never move hi outside
+// sigma_H >= (8 nd + 1) M^2 and is folded into a pair accumulator (and reset)
+// after every 4 sites, so its 4 nd terms never move hi outside
 // [sigma_H / 2, 2 sigma_H] and hi - sigma_H is exact.  A - sigma_A and
 // B - sigma_B are exact because sigma is a power of two no smaller than any
 // term and hi stays below 2^24 sigma.
@@ -128,12 +128,16 @@ __global__ void __launch_bounds__(kActThreads) action_kernel(int nd, int L, int 
 // The B term also needs the cross term 2 q qe of c^4 = (q + qe)^2 (q = fl(c c),
 // qe its FMA residual; qe^2 ~ 2^-48 q^2 is dropped), collected in plain FP32.
 //
-// The biased H accumulator keeps about 2^-47 sigma_H per fold.  When the
+// The biased H accumulator keeps about 2^-48 sigma_H per fold.  When the
 // field has a few sites far larger than the rest, sigma_H is large next to the
 // typical product and that is not enough: after the block sum, a
-// configuration whose estimated H error, 2^-44.5 sigma_H sqrt(V / 8), exceeds
+// configuration whose estimated H error, 2^-45.5 sigma_H sqrt(V / 4), exceeds
 // 1e-13 max(|S|, 1) is summed again from global memory with a general pair
-// sum per site (site_term_ff, as the non-streaming kernel does).
+// sum per site (site_term_ff, as the non-streaming kernel does).  That is slow,
+// so the folds are short: with a fold every 8 sites (sigma_H twice as large,
+// four times the error per fold) most configurations of a thermalised chain of
+// 3D L=16 (m2 = -6, lam = 5) were summed again: 418 us instead of 84 us for
+// 16,384 of them.
 //
 // Per configuration there is one block barrier: before it every thread
 // leaves its share of S (pairs combined with c2d, lam and -2) in shared memory
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(kAsThreads) action_stream_kernel(int64_t B, co
 #pragma unroll
         for (int w = 1; w < kAsWarps; ++w) M = fmaxf(M, wmax[slot * kAsWarps + w]);
         const float M2 = M * M;
-        const float sA = pow2_ceil(M2), sB = pow2_ceil(M2 * M2), sH = pow2_ceil((16.f * ND + 1.f) * M2);
+        const float sA = pow2_ceil(M2), sB = pow2_ceil(M2 * M2), sH = pow2_ceil((8.f * ND + 1.f) * M2);
 
         // A, B and H of this thread's chunks (see above); xB collects q qe,
         // the cross term of c^4 = (q + qe)^2 (qe^2 ~ 2^-48 q^2 is dropped)
@@ -271,11 +275,10 @@ __global__ void __launch_bounds__(kAsThreads) action_stream_kernel(int64_t B, co
                     if constexpr (ND == 3) f2s_prod(aH, lH, c, zs[j]);
                 }
             }
-            if ((i & 1) || i == ITER - 1) {     // fold H (hi - sigma_H is exact) and restart it
-                ff_add(hsum, FF{aH - sH, lH});
-                aH = sH;
-                lH = 0.f;
-            }
+            // fold H (hi - sigma_H is exact) and restart it
+            ff_add(hsum, FF{aH - sH, lH});
+            aH = sH;
+            lH = 0.f;
         }
         // this thread's share of S = c2d A + lam B - 2 H
         FF t = ff_mul(c2d_ff, FF{aA - sA, lA});
@@ -303,10 +306,10 @@ __global__ void __launch_bounds__(kAsThreads) action_stream_kernel(int64_t B, co
             for (int w = 1; w < kAsWarps; ++w) ff_add(tot, pk[lane + 32 * w]);
             tot = warp_sum_ff(tot);
             // statistical size of the biased H error against the tolerance:
-            // 2^-44.5 sqrt(V/8) sigma_H <= 1e-13 max(|S|, 1), else (or NaN) the
+            // 2^-45.5 sqrt(V/4) sigma_H <= 1e-13 max(|S|, 1), else (or NaN) the
             // warp sums the configuration again from global memory, a general
             // pair sum per site
-            const float h_err = sH * (0.42044820f * sqrtf((float)(V / 8)));
+            const float h_err = sH * (0.21022410f * sqrtf((float)(V / 4)));
             if (!(h_err <= fmaxf(fabsf(tot.hi), 1.f))) {
                 const float* g = phi + b * V;
                 FF a{0.f, 0.f};
