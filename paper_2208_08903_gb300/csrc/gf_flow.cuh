@@ -20,7 +20,7 @@ namespace gf {
 //                                          <- h2 of slices s0-1 .. s0+n in in[0..n+2)
 constexpr int PH_H1 = 0, PH_H2 = 1, PH_C3 = 2;
 constexpr int MAX_PHASE_SLICES = 62;
-constexpr int kF32Tiles = 7, kCtaSizes = 4;   // fused FP32 kernel: conv2 tiles; CTAs of 64 << i threads
+constexpr int kF32Tiles = 6, kCtaSizes = 4;   // fused FP32 kernel: conv2 tiles; CTAs of 64 << i threads
 
 struct Phase {
     uint8_t type, n;
@@ -80,7 +80,7 @@ struct gf_flow {
     // reverse pass: the weight gradients of a layer run on `side`, forked from
     // and joined back into the caller's stream with these events
     cudaStream_t side;
-    cudaEvent_t ev_fork[3], ev_join;
+    cudaEvent_t ev_fork[2], ev_join;
 };
 
 namespace gf {
@@ -115,6 +115,10 @@ gf_status launch_flow_fp32_c32(const gf_flow* f, bool inverse, const gf_phi4* ph
 bool fp32_c32_recompute_supported(const gf_flow* f);
 gf_status launch_c32_recompute(const gf_flow* f, int layer, int64_t B, const float* xl, float* h1_out, float* h2_out,
                                float* s_out, cudaStream_t stream);
+
+// The same for every flow of two equal hidden widths (gf_flow_fp32.cu).
+gf_status launch_recompute(const gf_flow* f, int layer, int64_t B, const float* xl, float* h1_out, float* h2_out,
+                           float* s_out, cudaStream_t stream);
 
 // Polls of the failure-path test hook of the tensor-core kernels
 // (gf_set_bf16_stall_test; 0 = off).

@@ -70,17 +70,20 @@ size_t plan_smem(const gf_flow* f, int R, int n_phases, bool gw, int stage_taps,
 // Cost model of a conv2 phase of n slices, in cycles per input channel: with
 // `resident` CTAs on an SM the FMA pipe (128 per cycle) or the shared-memory
 // reads (one 128-byte wavefront per cycle: NS for the sites, CO / 4 for the
-// weights) bound it; one CTA alone needs at least its warps' own issue time.
+// weights) bound it, plus the issue slots that pairing a site's value with itself
+// takes; one CTA alone needs its warps' issue time on the busiest of the four
+// schedulers and about 0.8 of a warp's for latencies that nothing hides.
 struct TileCost { double eff, lat; int passes; };
 TileCost tile_cost(int nf, int C, int tile, int warps) {
     const int ns = kTileNS[tile], co = kTileCO[tile];
     const int tasks = (nf + 32 * ns - 1) / (32 * ns) * (C / co);
     TileCost t;
     t.passes = (tasks + warps - 1) / warps;
-    t.eff = tasks * (std::max(ns * co / 4.0, ns + std::max(1.0, co / 4.0)) + 0.5);
+    t.eff = tasks * (std::max(ns * co / 4.0, ns + std::max(1.0, co / 4.0)) + 0.5 + 0.4 * ns);
+    const double c = ns * co + 1.6 * ns + 2.0;
     t.lat = 0;
     for (int left = tasks; left > 0; left -= warps)
-        t.lat += ((std::min(left, warps) + 3) / 4) * (ns * co + 2.0) + 8.0;
+        t.lat += ((std::min(left, warps) + 3) / 4 + 0.8) * c;
     return t;
 }
 // The conv2 phases of one layer with one tile.
@@ -147,7 +150,7 @@ gf_status flow_fp32_configure(gf_flow* f) {
     const int tap = C * C * 4;
     f->stage_taps = f->T * tap <= 12 * 1024 ? f->T : std::max(1, 8192 / tap);
     f->weights_global = false;
-    if (fp32_c32_supported(f)) {                         // (its own kernel: no plan needed)
+    if (fp32_c32_recompute_supported(f)) {               // (kernels of its own for everything: no plan needed)
         f->full = true; f->G = L; f->R = L; f->n_phases = 3;
         return GF_OK;
     }
@@ -193,17 +196,13 @@ gf_status flow_fp32_configure(gf_flow* f) {
     return GF_OK;
 }
 
-gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, int64_t B,
-                           uint64_t seed, uint64_t counter0, const float* z_in, float* z_out,
-                           const float* phi_in, float* phi_out, double* logq_out,
-                           double* S_out, double* logw_out, cudaStream_t stream, float* xs_out, int64_t xs_stride,
-                           double* logdet_out) {
-    if (fp32_c32_supported(f))
-        return launch_flow_fp32_c32(f, inverse, phi4, B, seed, counter0, z_in, z_out, phi_in, phi_out, logq_out,
-                                    S_out, logw_out, stream, xs_out, xs_stride, logdet_out);
+namespace {
+
+// Fills in the plan of a launch over a.B configurations, chooses its CTA size
+// and tile and launches it.
+gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t stream) {
+    const int64_t B = a.B;
     if (B <= 0) return GF_OK;
-    FlowArgs a;
-    std::memset(&a, 0, sizeof(a));
     const int L = f->shape.L, C = f->C1;
     const bool gw = f->weights_global;
     a.W = f->d_packed;
@@ -212,11 +211,10 @@ gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, 
     a.stride = f->packed_stride;
     a.off = packed_offsets(f->T, C, C);
     a.L = L; a.S = f->S; a.V = f->V;
-    a.n_layers = f->shape.n_layers; a.R = f->R;
+    a.R = f->R;
     a.stage_taps = f->stage_taps;
     a.n_stages = (f->T + f->stage_taps - 1) / f->stage_taps;
     a.two_small = f->two_small;
-    a.head_train = xs_out != nullptr;
     a.head_G = f->head_G;
     a.head_zb = a.head_train ? L : f->head_zb;
     a.head_a = a.head_train ? 1 : f->head_a;
@@ -227,13 +225,6 @@ gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, 
     a.fd_Lh = make_fastdiv((uint32_t)(L / 2));
     a.slope = (float)f->shape.leaky_slope;
     a.use_tanh = f->shape.use_final_tanh;
-    a.has_phi4 = phi4 != nullptr;
-    ff_split(2.0 * f->shape.nd + (phi4 ? phi4->m2 : 0.0), &a.c2d_ff.hi, &a.c2d_ff.lo);
-    ff_split(phi4 ? phi4->lam : 0.0, &a.lam_ff.hi, &a.lam_ff.lo);
-    a.B = B; a.seed = seed; a.counter0 = counter0;
-    a.z_in = z_in; a.z_out = z_out; a.phi_in = phi_in; a.phi_out = phi_out;
-    a.logq_out = logq_out; a.S_out = S_out; a.logw_out = logw_out;
-    a.xs_out = xs_out; a.xs_stride = xs_stride; a.logdet_out = logdet_out;
     const size_t smem = plan_smem(f, f->R, f->n_phases, gw, f->stage_taps, f->two_small, &a);
 
     // CTA size and tile: those that finish the batch soonest (estimated: conv2
@@ -248,7 +239,7 @@ gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, 
             const int nt = 64 << i, r = (int)std::min<int64_t>((B + sms - 1) / sms, ctas_per_sm(smem, nt));
             const TileCost c = layer_cost(f->h2_count, f->S, C, t, nt / 32);
             const double items = (double)f->V * (C / 8 * 2 + 2) / nt;            // conv1 and head items per thread
-            const double lat = c.lat * f->T * C + 2500.0 + 60.0 * f->T / 9 * items, eff = 1.2 * c.eff * f->T * C;
+            const double lat = c.lat * f->T * C + 2500.0 + 1.2 * nt + 60.0 * f->T / 9 * items, eff = 1.2 * c.eff * f->T * C;
             const double cost = (double)((B + sms * r - 1) / (sms * r)) * std::max(lat, r * eff);
             if (nti < 0 || cost < best) { best = cost; nti = i; tile = t; }
         }
@@ -259,6 +250,44 @@ gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, 
     kernel_for(f, tile)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
     GF_CHECK_LAUNCH();
     return GF_OK;
+}
+
+}  // namespace
+
+gf_status launch_flow_fp32(const gf_flow* f, bool inverse, const gf_phi4* phi4, int64_t B,
+                           uint64_t seed, uint64_t counter0, const float* z_in, float* z_out,
+                           const float* phi_in, float* phi_out, double* logq_out,
+                           double* S_out, double* logw_out, cudaStream_t stream, float* xs_out, int64_t xs_stride,
+                           double* logdet_out) {
+    if (fp32_c32_supported(f))
+        return launch_flow_fp32_c32(f, inverse, phi4, B, seed, counter0, z_in, z_out, phi_in, phi_out, logq_out,
+                                    S_out, logw_out, stream, xs_out, xs_stride, logdet_out);
+    FlowArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.n_layers = f->shape.n_layers;
+    a.head_train = xs_out != nullptr;
+    a.has_phi4 = phi4 != nullptr;
+    ff_split(2.0 * f->shape.nd + (phi4 ? phi4->m2 : 0.0), &a.c2d_ff.hi, &a.c2d_ff.lo);
+    ff_split(phi4 ? phi4->lam : 0.0, &a.lam_ff.hi, &a.lam_ff.lo);
+    a.B = B; a.seed = seed; a.counter0 = counter0;
+    a.z_in = z_in; a.z_out = z_out; a.phi_in = phi_in; a.phi_out = phi_out;
+    a.logq_out = logq_out; a.S_out = S_out; a.logw_out = logw_out;
+    a.xs_out = xs_out; a.xs_stride = xs_stride; a.logdet_out = logdet_out;
+    return launch_plan(f, a, inverse, stream);
+}
+
+gf_status launch_recompute(const gf_flow* f, int layer, int64_t B, const float* xl, float* h1_out, float* h2_out,
+                           float* s_out, cudaStream_t stream) {
+    if (fp32_c32_recompute_supported(f)) return launch_c32_recompute(f, layer, B, xl, h1_out, h2_out, s_out, stream);
+    FlowArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.layer0 = layer;
+    a.n_layers = 1;
+    a.head_train = 1;
+    a.B = B;
+    a.z_in = xl;
+    a.h1_out = h1_out; a.h2_out = h2_out; a.s_out = s_out;
+    return launch_plan(f, a, false, stream);
 }
 
 }  // namespace gf

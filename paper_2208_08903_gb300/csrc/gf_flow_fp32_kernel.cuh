@@ -51,7 +51,7 @@ struct FlowArgs {
     int n_phases, n_passes;    // n_passes: conv2 passes of one layer
     int64_t stride;
     PackedOffsets off;
-    int L, S, V, n_layers, R;
+    int L, S, V, layer0, n_layers, R;
     int stage_taps, n_stages;  // taps of W2 per staging buffer
     int two_small;             // second buffer for the layer's other weights
     int head_G, head_zb, head_a, head_b, head_train;   // see HeadSplit
@@ -71,14 +71,20 @@ struct FlowArgs {
     float* xs_out;             // training: the field after l layers at xs_out + l xs_stride + b V
     int64_t xs_stride;
     double* logdet_out;
+    // training's recompute of layer layer0 from its input (z_in), all three set:
+    // h1, h2 [B][C/4][V][4] and s [B][V] at the updated sites; nothing else
+    float* h1_out;
+    float* h2_out;
+    float* s_out;
     int off_h1, off_h2, off_small, off_w2, off_red, off_s, off_sched;   // shared memory (floats)
 };
 
 // conv2 tiles (sites per lane, output channels); the last is also the one of
-// the kernels that read their weights from global memory
+// the kernels that read their weights from global memory.  (16 channels per
+// tile need fewer loads per FMA but ran 5 % to 15 % slower at every shape.)
 constexpr int kTiles = kF32Tiles;
-constexpr int kTileNS[kTiles] = {1, 1, 2, 3, 5, 6, 4};
-constexpr int kTileCO[kTiles] = {2, 4, 8, 8, 8, 8, 8};
+constexpr int kTileNS[kTiles] = {1, 1, 2, 3, 5, 4};
+constexpr int kTileCO[kTiles] = {2, 4, 8, 8, 8, 8};
 constexpr int kTileGW = kTiles - 1;
 
 __device__ __forceinline__ int wrap(int v, int L) { return v < 0 ? v + L : (v >= L ? v - L : v); }
@@ -194,7 +200,7 @@ struct Weights {
 // reach fixed sites; the others add nothing).
 template <int ND, int C, bool GW>
 __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, const float* x, float* h1,
-                         int frozen) {
+                         int frozen, int64_t b) {
     const int L = a.L, S = a.S, hS = S >> 1, nf = ph.n * S, half = nf >> 1;
     const float* W1 = w.W1();
     const float* b1 = w.b1();
@@ -233,6 +239,11 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
         for (int i = 0; i < 4; ++i) { v[2 * i] = lrelu(f2_lo(acc[i]), a.slope); v[2 * i + 1] = lrelu(f2_hi(acc[i]), a.slope); }
         *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<float4*>(o + 4 * S) = make_float4(v[4], v[5], v[6], v[7]);
+        if (a.h1_out) {
+            float* go = a.h1_out + ((b * (C / 4) + 2 * g) * a.V + sl * S + (ND == 3 ? y * L : 0) + xc) * 4;
+            *reinterpret_cast<float4*>(go) = make_float4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<float4*>(go + 4 * (int64_t)a.V) = make_float4(v[4], v[5], v[6], v[7]);
+        }
     }
 }
 
@@ -240,7 +251,7 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
 // One pass: warp `task` = 32 NS consecutive sites of the phase x CO channels.
 template <int ND, int C, int NS, int CO, bool GW>
 __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>& w, const Phase& ph, const float* h1,
-                                        float* h2, int pass) {
+                                        float* h2, int pass, int64_t b) {
     const int L = a.L, S = a.S, nf = ph.n * S, nblk = (nf + 32 * NS - 1) / (32 * NS);
     const int lane = threadIdx.x & 31, task = pass * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
     const int g = task / nblk, blk = task - g * nblk, co = g * CO;
@@ -257,12 +268,12 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
         w.begin_stage(st);
         if (!active) continue;
         if (st == 0) {
-            f32x2 b[CO / 2];
-            load_w<CO, GW>(b, w.b2() + co);
+            f32x2 bias[CO / 2];
+            load_w<CO, GW>(bias, w.b2() + co);
 #pragma unroll
             for (int k = 0; k < NS; ++k)
 #pragma unroll
-                for (int i = 0; i < CO / 2; ++i) acc[k][i] = b[i];
+                for (int i = 0; i < CO / 2; ++i) acc[k][i] = bias[i];
         }
         const auto tap = [&](int t, int t0) {
             const int ds = ND == 3 ? t / 9 - 1 : t / 3 - 1, dy = ND == 3 ? (t / 3) % 3 - 1 : 0, dx = t % 3 - 1;
@@ -319,6 +330,13 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
             for (int i = 0; i < CO / 4; ++i)
                 *reinterpret_cast<float4*>(o + (size_t)i * S * 4) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
+        if (a.h2_out) {
+            const int n = wrap(ph.s0 + (at[k] >> 20), L) * S + (ND == 3 ? ((at[k] >> 10) & 1023) * L : 0) + (at[k] & 1023);
+            float* go = a.h2_out + ((b * (C / 4) + (co >> 2)) * a.V + n) * 4 + (co & 3);
+#pragma unroll
+            for (int i = 0; i < CO; i += 2)
+                *reinterpret_cast<float2*>(go + (int64_t)(i / 4) * a.V * 4 + (i & 3)) = make_float2(v[i], v[i + 1]);
+        }
     }
 }
 
@@ -328,7 +346,7 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
 // taps, combined with xor-shuffles.
 template <int ND, int C, bool GW>
 __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, int r0, int nr, int tps,
-                         const float* h2, float* x, float* s_site, int frozen, bool inverse, FF& logdet) {
+                         const float* h2, float* x, float* s_site, int frozen, bool inverse, FF& logdet, int64_t b) {
     constexpr int T = ND == 3 ? 27 : 9;
     const int L = a.L, S = a.S, half = S >> 1;
     const int lt = 31 - __clz(tps), nchunk = (C / 4) >> lt;
@@ -377,6 +395,10 @@ __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
             const float spre = a.head_train ? ps : ps + bs, tt = a.head_train ? pt : pt + bt;
             const float s = a.use_tanh ? tanhf(spre) : spre;
             const int n = sl * S + (ND == 3 ? y * L : 0) + xc;
+            if (a.s_out) {
+                a.s_out[b * a.V + n] = s;
+                continue;
+            }
             if (!inverse) x[n] = fmaf(x[n], expf(s), tt);
             else x[n] = (x[n] - tt) * expf(-s);
             if (GW) ff_add(logdet, s);             // (256 threads and the blocks of head_split: the same order)
@@ -439,7 +461,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             reinterpret_cast<uint32_t*>(smf + a.off_sched)[i] = __ldg(reinterpret_cast<const uint32_t*>(a.sched) + i);
     const int64_t n_cfg = a.B > (int64_t)blockIdx.x ? (a.B - 1 - (int64_t)blockIdx.x) / gridDim.x + 1 : 0;
     const int N = a.n_layers;
-    Weights<ND, C, GW> w{a, smf, n_cfg * N - 1, inverse ? N - 1 : 0, 0, 0, 0, 0, true};
+    Weights<ND, C, GW> w{a, smf, n_cfg * N - 1, inverse ? N - 1 : a.layer0, 0, 0, 0, 0, true};
     if (!GW && n_cfg * N > 0) {
         w.load_small(0, w.l);
         w.load_w2(0, w.l, 0);
@@ -477,7 +499,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             }
             return v;
         };
-        if (!inverse) {
+        if (!inverse && !a.s_out) {
             z2 = order_sum(red, sum_squares);
             for (int n = threadIdx.x; n < V; n += blockDim.x) {
                 const float v = x[n];
@@ -487,7 +509,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
         }
 
         for (int li = 0; li < N; ++li) {
-            w.lnext = inverse ? (w.l == 0 ? N - 1 : w.l - 1) : (w.l + 1 == N ? 0 : w.l + 1);
+            w.lnext = inverse ? (w.l == 0 ? N - 1 : w.l - 1) : (w.l + 1 == a.layer0 + N ? a.layer0 : w.l + 1);
             const int frozen = w.l & 1;
             if (a.xs_out && li > 0) {
                 __syncthreads();
@@ -499,18 +521,18 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
                 const Phase& ph = sched[p];
                 if (ph.type == PH_H2) {            // begins with a barrier of its own (begin_stage)
                     const int tasks = ((ph.n * a.S + 32 * NS - 1) / (32 * NS)) * (C / CO), nw = (int)(blockDim.x >> 5);
-                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW>(a, w, ph, h1, h2, q);
+                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW>(a, w, ph, h1, h2, q, b);
                     continue;
                 }
                 __syncthreads();
                 if (ph.type == PH_H1) {
                     if (!GW && p == 0 && li > 0) add_logdet(a, s_site, logdet);
-                    phase_h1<ND, C, GW>(a, w, ph, x, h1, frozen);
+                    phase_h1<ND, C, GW>(a, w, ph, x, h1, frozen, b);
                 } else {
                     const int na = max(0, min((int)ph.n, a.head_zb - (int)ph.s0));
-                    if (na > 0) phase_c3<ND, C, GW>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0]);
+                    if (na > 0) phase_c3<ND, C, GW>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0], b);
                     if (na < ph.n)
-                        phase_c3<ND, C, GW>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0]);
+                        phase_c3<ND, C, GW>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0], b);
                 }
             }
             w.end_layer();
@@ -518,6 +540,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             --w.left;
         }
         __syncthreads();
+        if (a.s_out) continue;                     // (uniform; the next configuration's x may be written now)
 
         for (int n = threadIdx.x; n < V; n += blockDim.x) {
             if (!inverse) a.phi_out[b * V + n] = x[n];
