@@ -20,6 +20,7 @@ namespace gf {
 //                                          <- h2 of slices s0-1 .. s0+n in in[0..n+2)
 constexpr int PH_H1 = 0, PH_H2 = 1, PH_C3 = 2;
 constexpr int MAX_PHASE_SLICES = 62;
+constexpr int kMaxPhaseKinds = 8;             // different slice counts of a layer's conv2 phases
 constexpr int kF32Tiles = 6, kCtaSizes = 4;   // fused FP32 kernel: conv2 tiles; CTAs of 64 << i threads
 
 struct Phase {
@@ -54,11 +55,13 @@ struct gf_flow {
     size_t smem_bytes;
     // fused FP32 kernel (gf_flow_fp32.cu): staged taps of W2 per buffer, a
     // second buffer for the other weights, or weights read from global memory;
-    // lanes per site of the head's sums; conv2 phases of a layer by slice count
+    // lanes per site of the head's sums; the conv2 phases of a layer: how many
+    // (h2_count[i]) of h2_n[i] slices
     int stage_taps;
     bool two_small, weights_global;
     int head_G, head_zb, head_a, head_b;
-    int16_t h2_count[gf::MAX_PHASE_SLICES + 1];
+    int n_h2;
+    int16_t h2_n[gf::kMaxPhaseKinds], h2_count[gf::kMaxPhaseKinds];
     // BF16 tensor-core path: the 3D L=16, C=32 kernel (gf_flow_bf16.cu) or,
     // when tc is set, the kernel for other shapes (gf_flow_tc.cu)
     void* d_bf16;           // per-layer weight blocks of the tensor-core kernel

@@ -72,9 +72,11 @@ size_t plan_smem(const gf_flow* f, int R, int n_phases, bool gw, int stage_taps,
 // reads (one 128-byte wavefront per cycle: NS for the sites, CO / 4 for the
 // weights) bound it, plus the issue slots that pairing a site's value with itself
 // takes; one CTA alone needs its warps' issue time on the busiest of the four
-// schedulers and about 0.8 of a warp's for latencies that nothing hides.
+// schedulers and, per pass, the latencies that nothing hides: about 20 cycles
+// and 0.4 of a warp's time, and no less than the arrival of a stage of weights
+// (800 cycles) over its `stage` channels.
 struct TileCost { double eff, lat; int passes; };
-TileCost tile_cost(int nf, int C, int tile, int warps) {
+TileCost tile_cost(int nf, int C, int tile, int warps, int stage) {
     const int ns = kTileNS[tile], co = kTileCO[tile];
     const int tasks = (nf + 32 * ns - 1) / (32 * ns) * (C / co);
     TileCost t;
@@ -83,38 +85,45 @@ TileCost tile_cost(int nf, int C, int tile, int warps) {
     const double c = ns * co + 1.6 * ns + 2.0;
     t.lat = 0;
     for (int left = tasks; left > 0; left -= warps)
-        t.lat += ((std::min(left, warps) + 3) / 4 + 0.8) * c;
+        t.lat += std::max(((std::min(left, warps) + 3) / 4 + 0.4) * c + 20.0, 800.0 / stage);
     return t;
 }
 // The conv2 phases of one layer with one tile.
-TileCost layer_cost(const int16_t* h2_count, int S, int C, int tile, int warps) {
+TileCost layer_cost(const gf_flow* f, int tile, int warps, int taps) {
     TileCost sum{0, 0, 0};
-    for (int n = 1; n <= MAX_PHASE_SLICES; ++n) {
-        if (!h2_count[n]) continue;
-        const TileCost t = tile_cost(n * S, C, tile, warps);
-        sum.eff += h2_count[n] * t.eff;
-        sum.lat += h2_count[n] * t.lat;
-        sum.passes += h2_count[n] * t.passes;
+    for (int i = 0; i < f->n_h2; ++i) {
+        const TileCost t = tile_cost(f->h2_n[i] * f->S, f->C1, tile, warps, taps * f->C1);
+        sum.eff += f->h2_count[i] * t.eff;
+        sum.lat += f->h2_count[i] * t.lat;
+        sum.passes += f->h2_count[i] * t.passes;
     }
     return sum;
 }
-void count_h2(const std::vector<Phase>& s, int16_t* h2_count) {
-    std::memset(h2_count, 0, sizeof(int16_t) * (MAX_PHASE_SLICES + 1));
-    for (const Phase& p : s)
-        if (p.type == PH_H2) ++h2_count[p.n];
+// Sets the flow's list of conv2 phases (false: more kinds than it holds).
+bool set_h2(gf_flow* f, const std::vector<Phase>& s) {
+    f->n_h2 = 0;
+    for (const Phase& p : s) {
+        if (p.type != PH_H2) continue;
+        int i = 0;
+        while (i < f->n_h2 && f->h2_n[i] != p.n) ++i;
+        if (i == kMaxPhaseKinds) return false;
+        if (i == f->n_h2) { f->h2_n[i] = p.n; f->h2_count[i] = 0; ++f->n_h2; }
+        ++f->h2_count[i];
+    }
+    return true;
 }
 
-FlowKernel kernel_for(const gf_flow* f, int tile) {
+FlowKernel kernel_for(const gf_flow* f, int tile, bool rec) {
     const bool gw = f->weights_global;
     switch (f->shape.nd * 100 + f->C1) {
-        case 208: return kernel_of<2, 8>(tile, gw);
-        case 216: return kernel_of<2, 16>(tile, gw);
-        case 224: return kernel_of<2, 24>(tile, gw);
-        case 232: return kernel_of<2, 32>(tile, gw);
-        case 308: return kernel_of<3, 8>(tile, gw);
-        case 316: return kernel_of<3, 16>(tile, gw);
-        case 324: return kernel_of<3, 24>(tile, gw);
-        default: return kernel_of<3, 32>(tile, gw);
+        case 208: return kernel_of<2, 8>(tile, gw, rec);
+        case 216: return kernel_of<2, 16>(tile, gw, rec);
+        case 224: return kernel_of<2, 24>(tile, gw, rec);
+        case 232: return kernel_of<2, 32>(tile, gw, rec);
+        case 308: return kernel_of<3, 8>(tile, gw, rec);
+        case 316: return kernel_of<3, 16>(tile, gw, rec);
+        case 324: return kernel_of<3, 24>(tile, gw, rec);
+        default: return kernel_of<3, 32>(tile, gw, rec);
     }
 }
 
@@ -158,7 +167,7 @@ gf_status flow_fp32_configure(gf_flow* f) {
     if (L <= MAX_PHASE_SLICES && plan_smem(f, L, 3, false, f->stage_taps, true, nullptr) <= kBudget) {
         f->full = true; f->two_small = true; f->G = L; f->R = L; f->n_phases = 3;
         f->smem_bytes = plan_smem(f, f->R, f->n_phases, false, f->stage_taps, true, nullptr);
-        f->h2_count[L] = 1;
+        f->n_h2 = 1; f->h2_n[0] = (int16_t)L; f->h2_count[0] = 1;
         return GF_OK;
     }
     // else G slices at a time: the cheapest G that fits, staging one tap per
@@ -170,18 +179,31 @@ gf_status flow_fp32_configure(gf_flow* f) {
         int top = std::min(MAX_PHASE_SLICES, L - 3);
         while (top >= 1 && plan_smem(f, top + 2, 0, false, taps, false, nullptr) > kBudget) --top;
         for (int G = top; G >= std::max(1, top - 7); --G) {
-            const std::vector<Phase> s = build_schedule(L, G, false);
-            if (plan_smem(f, G + 2, (int)s.size(), false, taps, false, nullptr) > kBudget) continue;
-            int16_t count[MAX_PHASE_SLICES + 1];
-            count_h2(s, count);
+            // the schedule's conv2 phases: the first block needs two slices more
+            // than it has, a short last one finds two in the cache
+            f->n_h2 = 0;
+            const auto add = [&](int n) {
+                int i = 0;
+                while (i < f->n_h2 && f->h2_n[i] != n) ++i;
+                if (i == f->n_h2) { f->h2_n[i] = (int16_t)n; f->h2_count[i] = 0; ++f->n_h2; }
+                ++f->h2_count[i];
+            };
+            for (int extra = 2; extra > 0; extra -= G) add(std::min(G, extra));
+            for (int a = 0; a < L; a += G)
+                if (L - a >= G) add(G);
+                else if (L - a > 2) add(L - a - 2);
             double c = 0;
             for (int t = 0; t < kTiles; ++t) {
-                const TileCost tc = layer_cost(count, f->S, C, t, 16);
-                const double ct = std::max(tc.eff, tc.lat) + 4.0 * s.size();     // phase overhead: barriers, tails
+                const TileCost tc = layer_cost(f, t, 16, taps);
+                const double ct = std::max(tc.eff, tc.lat) + 12.0 * ((L + G - 1) / G + 1);   // phase overhead: barriers, tails
                 if (c == 0 || ct < c) c = ct;
             }
-            if (!bestG || c < 0.98 * best) { best = c; bestG = G; best_taps = taps; best_phases = (int)s.size(); }
+            if (bestG && c >= 0.98 * best) continue;
+            const int phases = (int)build_schedule(L, G, false).size();
+            if (plan_smem(f, G + 2, phases, false, taps, false, nullptr) > kBudget) continue;
+            best = c; bestG = G; best_taps = taps; best_phases = phases;
         }
+        if (taps == 1) break;
     }
     if (!bestG) {                                        // weights read from global memory
         f->weights_global = true;
@@ -192,8 +214,7 @@ gf_status flow_fp32_configure(gf_flow* f) {
     }
     f->G = bestG; f->R = bestG + 2; f->stage_taps = best_taps; f->n_phases = best_phases;
     f->smem_bytes = plan_smem(f, f->R, f->n_phases, f->weights_global, best_taps, false, nullptr);
-    count_h2(build_schedule(L, f->G, false), f->h2_count);
-    return GF_OK;
+    return set_h2(f, build_schedule(L, f->G, false)) ? GF_OK : GF_EUNSUPPORTED;
 }
 
 namespace {
@@ -204,7 +225,8 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
     const int64_t B = a.B;
     if (B <= 0) return GF_OK;
     const int L = f->shape.L, C = f->C1;
-    const bool gw = f->weights_global;
+    const bool gw = f->weights_global, rec = a.s_out != nullptr;
+    if (gw && rec) return GF_EUNSUPPORTED;
     a.W = f->d_packed;
     a.sched = f->d_sched;
     a.n_phases = f->n_phases;
@@ -234,20 +256,20 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
     int nti = -1, tile = 0;
     const int64_t sms = num_sms();
     double best = 0;
-    for (int t = gw ? kTileGW : 0; t < kTiles; ++t)
+    for (int t = gw ? kTileGW : rec ? kTileRec : 0; t < kTiles; ++t)
         for (int i = gw ? kCtaSizes - 2 : f->full ? 0 : kCtaSizes - 1; i < (gw ? kCtaSizes - 1 : kCtaSizes); ++i) {
             const int nt = 64 << i, r = (int)std::min<int64_t>((B + sms - 1) / sms, ctas_per_sm(smem, nt));
-            const TileCost c = layer_cost(f->h2_count, f->S, C, t, nt / 32);
+            const TileCost c = layer_cost(f, t, nt / 32, f->stage_taps);
             const double items = (double)f->V * (C / 8 * 2 + 2) / nt;            // conv1 and head items per thread
             const double lat = c.lat * f->T * C + 2500.0 + 1.2 * nt + 60.0 * f->T / 9 * items, eff = 1.2 * c.eff * f->T * C;
             const double cost = (double)((B + sms * r - 1) / (sms * r)) * std::max(lat, r * eff);
             if (nti < 0 || cost < best) { best = cost; nti = i; tile = t; }
         }
-    if (nti < 0 || !allow_smem(kernel_for(f, tile))) return GF_ECUDA;
+    if (nti < 0 || !allow_smem(kernel_for(f, tile, rec))) return GF_ECUDA;
     const int NT = 64 << nti;
-    a.n_passes = layer_cost(f->h2_count, f->S, C, tile, NT / 32).passes;
+    a.n_passes = layer_cost(f, tile, NT / 32, f->stage_taps).passes;
     const int64_t grid = std::min<int64_t>(B, sms * ctas_per_sm(smem, NT));
-    kernel_for(f, tile)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
+    kernel_for(f, tile, rec)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
     GF_CHECK_LAUNCH();
     return GF_OK;
 }

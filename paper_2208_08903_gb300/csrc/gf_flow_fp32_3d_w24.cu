@@ -5,7 +5,7 @@ namespace gf {
 namespace f32k {
 
 template <>
-FlowKernel kernel_of<3, 24>(int tile, bool gw) { return pick_kernel<3, 24>(tile, gw); }
+FlowKernel kernel_of<3, 24>(int tile, bool gw, bool rec) { return pick_kernel<3, 24>(tile, gw, rec); }
 
 }  // namespace f32k
 }  // namespace gf

@@ -198,7 +198,7 @@ struct Weights {
 // h1 = LReLU(conv1(x at the sites of parity `frozen`)), 8 channels per thread,
 // sites ordered by parity so that a warp's live taps agree (half of the taps
 // reach fixed sites; the others add nothing).
-template <int ND, int C, bool GW>
+template <int ND, int C, bool GW, bool REC>
 __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, const float* x, float* h1,
                          int frozen, int64_t b) {
     const int L = a.L, S = a.S, hS = S >> 1, nf = ph.n * S, half = nf >> 1;
@@ -239,7 +239,7 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
         for (int i = 0; i < 4; ++i) { v[2 * i] = lrelu(f2_lo(acc[i]), a.slope); v[2 * i + 1] = lrelu(f2_hi(acc[i]), a.slope); }
         *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<float4*>(o + 4 * S) = make_float4(v[4], v[5], v[6], v[7]);
-        if (a.h1_out) {
+        if constexpr (REC) {
             float* go = a.h1_out + ((b * (C / 4) + 2 * g) * a.V + sl * S + (ND == 3 ? y * L : 0) + xc) * 4;
             *reinterpret_cast<float4*>(go) = make_float4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<float4*>(go + 4 * (int64_t)a.V) = make_float4(v[4], v[5], v[6], v[7]);
@@ -249,7 +249,7 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
 
 // ---------------------------------------------------------------- conv2
 // One pass: warp `task` = 32 NS consecutive sites of the phase x CO channels.
-template <int ND, int C, int NS, int CO, bool GW>
+template <int ND, int C, int NS, int CO, bool GW, bool REC>
 __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>& w, const Phase& ph, const float* h1,
                                         float* h2, int pass, int64_t b) {
     const int L = a.L, S = a.S, nf = ph.n * S, nblk = (nf + 32 * NS - 1) / (32 * NS);
@@ -330,7 +330,7 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
             for (int i = 0; i < CO / 4; ++i)
                 *reinterpret_cast<float4*>(o + (size_t)i * S * 4) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
-        if (a.h2_out) {
+        if constexpr (REC) {
             const int n = wrap(ph.s0 + (at[k] >> 20), L) * S + (ND == 3 ? ((at[k] >> 10) & 1023) * L : 0) + (at[k] & 1023);
             float* go = a.h2_out + ((b * (C / 4) + (co >> 2)) * a.V + n) * 4 + (co & 3);
 #pragma unroll
@@ -344,7 +344,7 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
 // (s, t) at the updated sites of slices r0 .. r0 + nr - 1 of the phase as one
 // packed pair; `tps` lanes share a site, each summing C / tps channels over all
 // taps, combined with xor-shuffles.
-template <int ND, int C, bool GW>
+template <int ND, int C, bool GW, bool REC>
 __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, int r0, int nr, int tps,
                          const float* h2, float* x, float* s_site, int frozen, bool inverse, FF& logdet, int64_t b) {
     constexpr int T = ND == 3 ? 27 : 9;
@@ -395,7 +395,7 @@ __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
             const float spre = a.head_train ? ps : ps + bs, tt = a.head_train ? pt : pt + bt;
             const float s = a.use_tanh ? tanhf(spre) : spre;
             const int n = sl * S + (ND == 3 ? y * L : 0) + xc;
-            if (a.s_out) {
+            if constexpr (REC) {
                 a.s_out[b * a.V + n] = s;
                 continue;
             }
@@ -446,7 +446,8 @@ __device__ double order_sum(FF* red, F part) {
     return ff_to_double(r);
 }
 
-template <int ND, int C, int NS, int CO, bool GW>
+// REC: training's recompute of one layer (h1_out, h2_out, s_out)
+template <int ND, int C, int NS, int CO, bool GW, bool REC>
 __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant__ FlowArgs a, int inverse) {
     extern __shared__ __align__(16) float smf[];
     const int V = a.V;
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             }
             return v;
         };
-        if (!inverse && !a.s_out) {
+        if (!inverse && !REC) {
             z2 = order_sum(red, sum_squares);
             for (int n = threadIdx.x; n < V; n += blockDim.x) {
                 const float v = x[n];
@@ -521,18 +522,18 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
                 const Phase& ph = sched[p];
                 if (ph.type == PH_H2) {            // begins with a barrier of its own (begin_stage)
                     const int tasks = ((ph.n * a.S + 32 * NS - 1) / (32 * NS)) * (C / CO), nw = (int)(blockDim.x >> 5);
-                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW>(a, w, ph, h1, h2, q, b);
+                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW, REC>(a, w, ph, h1, h2, q, b);
                     continue;
                 }
                 __syncthreads();
                 if (ph.type == PH_H1) {
                     if (!GW && p == 0 && li > 0) add_logdet(a, s_site, logdet);
-                    phase_h1<ND, C, GW>(a, w, ph, x, h1, frozen, b);
+                    phase_h1<ND, C, GW, REC>(a, w, ph, x, h1, frozen, b);
                 } else {
                     const int na = max(0, min((int)ph.n, a.head_zb - (int)ph.s0));
-                    if (na > 0) phase_c3<ND, C, GW>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0], b);
+                    if (na > 0) phase_c3<ND, C, GW, REC>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0], b);
                     if (na < ph.n)
-                        phase_c3<ND, C, GW>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0], b);
+                        phase_c3<ND, C, GW, REC>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0], b);
                 }
             }
             w.end_layer();
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             --w.left;
         }
         __syncthreads();
-        if (a.s_out) continue;                     // (uniform; the next configuration's x may be written now)
+        if constexpr (REC) continue;               // ( the next configuration's x may be written now)
 
         for (int n = threadIdx.x; n < V; n += blockDim.x) {
             if (!inverse) a.phi_out[b * V + n] = x[n];
@@ -568,18 +569,22 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
 }
 
 using FlowKernel = void (*)(const FlowArgs, int);
-// the kernel of a lattice dimension, width and tile (gf_flow_fp32_c*.cu)
+// the kernel of a lattice dimension, width and tile (gf_flow_fp32_*d_w*.cu);
+// recompute: tiles from kTileRec on
+constexpr int kTileRec = 2;
 template <int ND, int C>
-FlowKernel kernel_of(int tile, bool gw);
+FlowKernel kernel_of(int tile, bool gw, bool rec);
 
 template <int ND, int C, int I = 0>
-FlowKernel pick_kernel(int tile, bool gw) {
+FlowKernel pick_kernel(int tile, bool gw, bool rec) {
     if constexpr (I == kTiles) {
         return nullptr;
     } else {
-        if (gw) return flow_fp32_kernel<ND, C, kTileNS[kTileGW], kTileCO[kTileGW], true>;
-        if (tile == I) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false>;
-        return pick_kernel<ND, C, I + 1>(tile, gw);
+        if (gw) return flow_fp32_kernel<ND, C, kTileNS[kTileGW], kTileCO[kTileGW], true, false>;
+        if (tile == I && !rec) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, false>;
+        if constexpr (I >= kTileRec)
+            if (tile == I && rec) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, true>;
+        return pick_kernel<ND, C, I + 1>(tile, gw, rec);
     }
 }
 
