@@ -40,11 +40,12 @@
 // 8 TMEM lanes (width-8 shuffles).  Per layer, with a barrier of the
 // configuration's warps between the phases:
 //   conv1 (all warps): h1 = LReLU(W1 * masked x + b1) at every site, BF16, at
-//     its padded position and at its periodic images;
-//   conv2 (two issuing threads on different sub-partitions, alternate tiles):
-//     two groups of four epilogue warps (one warp per TMEM lane quarter) take
-//     the same alternate tiles, each through its own ring of TMEM
-//     accumulators, and turn them into
+//     its padded position and at its periodic images (or those by a pass of
+//     their own);
+//   conv2 (NG issuing threads, one per sub-partition, every NG-th tile each):
+//     NG groups of four epilogue warps (one warp per TMEM lane quarter) take
+//     the same tiles, each through its own ring of TMEM accumulators, and turn
+//     them into
 //     h2 = LReLU(acc + b2) in FP16, released from TMEM at once and written
 //     over h1 in place once every tile that reads those positions (up to
 //     ceil(p0 / 96) tiles on, p0 = 1 + P (+ P^2) the largest tap offset) has
@@ -62,11 +63,13 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "gf_async.cuh"
+#include "gf_f32x2.cuh"
 #include "gf_flow.cuh"
 #include "gf_tcgen05.cuh"
 
@@ -74,10 +77,15 @@ namespace gf {
 
 namespace {
 
-constexpr int kTcThreads = 384;           // warps 0, 1: MMA issue (warp 0 owns TMEM); warps 4..11: two epilogue groups
+// A configuration's warps: 0 .. NG-1 issue MMAs (warp 0 owns TMEM), 4 .. 4 NG + 3
+// are NG epilogue groups of four.  NG = 2 where two configurations can share a
+// CTA, 4 where one fills it (a single configuration's 12 warps left the SM at
+// 45 % issue, waiting for one another: see flow_tc_kernel).
+template <int NG>
+__host__ __device__ constexpr int tc_threads() { return 128 + 128 * NG; }
 constexpr int kTcM = 128;                 // rows per tile (TMEM lanes)
 constexpr int kTcOut = 96;                // output positions per tile (6 of every 8 rows)
-constexpr int kTcRing = 8;                // TMEM accumulators per epilogue group (at most)
+constexpr int kTcRings = 16;              // TMEM accumulators of all epilogue groups (at most)
 constexpr int kTcMaxTiles = 64;           // tiles per layer (one completion barrier each)
 constexpr long long kTcWaitLimit = 1ll << 22;
 constexpr int kSmemPerCTA = 232448;       // 227 KB opt-in maximum per CTA
@@ -126,7 +134,6 @@ __host__ __device__ inline int tc8_tap(int nd, int k, int kh) {
     if (kh == 0 && ta == (nd == 3 ? 7 : 1) && k == (nd == 3 ? 4 : 1)) return -1;
     return ta + kh;
 }
-__device__ __forceinline__ float lrelu_tc(float v, float a) { return v > 0.f ? v : a * v; }
 
 // Bounded wait for completion number n (0-based) of an mbarrier (phase parity
 // n & 1; every waiter has seen completion n - 1 already, so the parity names
@@ -178,22 +185,57 @@ __device__ __forceinline__ void pos_xyz(int p, int P, int PP, FastDiv fdP, FastD
     px = rem - py * P;
 }
 
-// conv1: h1 = LReLU(W1 * (x at the frozen sites) + b1) for every site, all
-// channels per thread, BF16, at the site's padded position and its periodic
-// images.  Sites are ordered (parity, site), so a warp holds one site parity
-// and the live taps (those that reach frozen sites) are the same for the
-// whole warp; the weight loads are broadcasts.  A thread takes NS sites of
-// one parity (j and j + V/(2 NS)), so each weight load feeds NS sites.  Site
-// j of parity q (rows y + L z in order, x fastest in a row): x = 2 (j mod
-// L/2) + ((q + y + z) mod 2).
-template <int ND, int CP, int NS>
+// LReLU of packed pairs: max(v, a v) for slopes a <= 1, the smaller of the two
+// above (the same numbers as v > 0 ? v : a v, in half the instructions).
+template <int N>
+__device__ __forceinline__ void lrelu_pairs(const f32x2 (&v)[N], f32x2 slope2, float* out) {
+    f32x2 av[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) av[i] = f2_mul(v[i], slope2);
+    if (f2_lo(slope2) <= 1.f) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            out[2 * i] = fmaxf(f2_lo(v[i]), f2_lo(av[i]));
+            out[2 * i + 1] = fmaxf(f2_hi(v[i]), f2_hi(av[i]));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            out[2 * i] = fminf(f2_lo(v[i]), f2_lo(av[i]));
+            out[2 * i + 1] = fminf(f2_hi(v[i]), f2_hi(av[i]));
+        }
+    }
+}
+// N/2 pairs from shared memory (16-byte aligned)
+template <int N>
+__device__ __forceinline__ void load_pairs(f32x2 (&w)[N / 2], const float* p) {
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) {
+        const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(p + 4 * i);
+        w[2 * i] = u.x;
+        w[2 * i + 1] = u.y;
+    }
+}
+
+// conv1: h1 = LReLU(W1 * (x at the frozen sites) + b1) for every site, BF16, at
+// the site's padded position and its periodic images.  Sites are ordered
+// (parity, site), so a warp holds one site parity (V a multiple of 128) and the
+// live taps (those that reach frozen sites) are the same for the whole warp; the
+// weight loads are broadcasts.  A thread takes NS sites of one parity (j and
+// j + V/(2 NS)) and CH of the channels, so each weight load feeds NS sites, as
+// packed FMAs over channel pairs.  Site j of parity q (rows y + L z in order, x
+// fastest in a row): x = 2 (j mod L/2) + ((q + y + z) mod 2).
+template <int ND, int CP, int NS, int CH, bool IMAGES>
 __device__ void tc_conv1(const TcGeom& g, const float* wf, const float* x, int frozen, float slope,
                          unsigned char* act, int t0, int nthr) {
-    constexpr int NKG = CP / 8;
     const int L = g.L, half = g.V >> 1, per = half / NS, Lh = L >> 1, P = g.P, npos = g.npos;
-    const float* W1 = wf + g.wf_W1;
-    const float* b1 = wf + g.wf_b1;
-    for (int it = t0; it < 2 * per; it += nthr) {
+    const f32x2 slope2 = f2_splat(slope);
+    for (int it0 = t0; it0 < 2 * per * (CP / CH); it0 += nthr) {
+        int cb = 0, it = it0;
+#pragma unroll
+        for (int k = 1; k < CP / CH; ++k)
+            if (it >= 2 * per) { it -= 2 * per; ++cb; }
+        const float* W1 = wf + g.wf_W1 + cb * CH;
         const int q = it >= per ? 1 : 0, j0 = it - q * per;
         int xc[NS], yc[NS], zc[NS], xs[NS][3], ys[NS][3], zs[NS][3];
 #pragma unroll
@@ -212,15 +254,12 @@ __device__ void tc_conv1(const TcGeom& g, const float* wf, const float* x, int f
                 zs[n][2] = wrapc(zc[n] + 1, L) * L * L;
             }
         }
-        float acc[NS][CP];
+        f32x2 acc[NS][CH / 2];
+        load_pairs<CH>(acc[0], wf + g.wf_b1 + cb * CH);
 #pragma unroll
-        for (int c4 = 0; c4 < CP / 4; ++c4) {
-            const float4 b = *reinterpret_cast<const float4*>(b1 + 4 * c4);
+        for (int n = 1; n < NS; ++n)
 #pragma unroll
-            for (int n = 0; n < NS; ++n) {
-                acc[n][4 * c4] = b.x; acc[n][4 * c4 + 1] = b.y; acc[n][4 * c4 + 2] = b.z; acc[n][4 * c4 + 3] = b.w;
-            }
-        }
+            for (int c = 0; c < CH / 2; ++c) acc[n][c] = acc[0][c];
 #pragma unroll
         for (int dz = 0; dz < (ND == 3 ? 3 : 1); ++dz) {
 #pragma unroll
@@ -231,47 +270,46 @@ __device__ void tc_conv1(const TcGeom& g, const float* wf, const float* x, int f
                     const int po = ND == 3 ? ((dx + dy + dz + 1) & 1) : ((dx + dy) & 1);
                     if ((q ^ po) != frozen) continue;
                     const int t = ND == 3 ? (dz * 3 + dy) * 3 + dx : dy * 3 + dx;
-                    float v[NS];
+                    f32x2 v[NS], w[CH / 2];
 #pragma unroll
-                    for (int n = 0; n < NS; ++n) v[n] = x[zs[n][dz] + ys[n][dy] + xs[n][dx]];
-                    const float4* w = reinterpret_cast<const float4*>(W1 + t * CP);
+                    for (int n = 0; n < NS; ++n) v[n] = f2_splat(x[zs[n][dz] + ys[n][dy] + xs[n][dx]]);
+                    load_pairs<CH>(w, W1 + t * CP);
 #pragma unroll
-                    for (int c4 = 0; c4 < CP / 4; ++c4) {
-                        const float4 ww = w[c4];
+                    for (int c = 0; c < CH / 2; ++c)
 #pragma unroll
-                        for (int n = 0; n < NS; ++n) {
-                            acc[n][4 * c4] = fmaf(v[n], ww.x, acc[n][4 * c4]);
-                            acc[n][4 * c4 + 1] = fmaf(v[n], ww.y, acc[n][4 * c4 + 1]);
-                            acc[n][4 * c4 + 2] = fmaf(v[n], ww.z, acc[n][4 * c4 + 2]);
-                            acc[n][4 * c4 + 3] = fmaf(v[n], ww.w, acc[n][4 * c4 + 3]);
-                        }
-                    }
+                        for (int n = 0; n < NS; ++n) acc[n][c] = f2_fma(v[n], w[c], acc[n][c]);
                 }
             }
         }
 #pragma unroll
         for (int n = 0; n < NS; ++n) {
+            float h[CH];
+            lrelu_pairs(acc[n], slope2, h);
+            // the site's padded position and, for a site on the first or last row of
+            // an axis, its images beyond the other end (byte offsets; predicated
+            // stores: loops over the images, as many as each site has, took longer
+            // than conv1 itself)
+            const int dx = (xc[n] == 0 ? L : xc[n] == L - 1 ? -L : 0) * 16;
+            const int dy = (yc[n] == 0 ? L : yc[n] == L - 1 ? -L : 0) * P * 16;
+            const int dz = ND == 3 ? (zc[n] == 0 ? L : zc[n] == L - 1 ? -L : 0) * P * P * 16 : 0;
+            unsigned char* at = act + (size_t)(cb * (CH / 8) * npos + xc[n] + 1 + (yc[n] + 1) * P +
+                                               (ND == 3 ? (zc[n] + 1) * P * P : 0)) * 16;
 #pragma unroll
-            for (int c = 0; c < CP; ++c) acc[n][c] = lrelu_tc(acc[n][c], slope);
-            // padded coordinates of the site and of its periodic images (a site on
-            // the first or last row of an axis is also the halo beyond the other end)
-            int xo[2], yo[2], zo[2], nx = 1, ny = 1, nz = 1;
-            xo[0] = xc[n] + 1;
-            if (xc[n] == 0) xo[nx++] = L + 1; else if (xc[n] == L - 1) xo[nx++] = 0;
-            yo[0] = (yc[n] + 1) * P;
-            if (yc[n] == 0) yo[ny++] = (L + 1) * P; else if (yc[n] == L - 1) yo[ny++] = 0;
-            zo[0] = ND == 3 ? (zc[n] + 1) * P * P : 0;
-            if (ND == 3) {
-                if (zc[n] == 0) zo[nz++] = (L + 1) * P * P; else if (zc[n] == L - 1) zo[nz++] = 0;
-            }
-#pragma unroll
-            for (int kg = 0; kg < NKG; ++kg) {
-                const uint4 w = pack_bf16x8(acc[n] + 8 * kg);
-                unsigned char* base = act + (size_t)kg * npos * 16;
-                for (int iz = 0; iz < nz; ++iz)
-                    for (int iy = 0; iy < ny; ++iy)
-                        for (int ix = 0; ix < nx; ++ix)
-                            *reinterpret_cast<uint4*>(base + (size_t)(xo[ix] + yo[iy] + zo[iz]) * 16) = w;
+            for (int kg = 0; kg < CH / 8; ++kg) {
+                const uint4 w = pack_bf16x8(h + 8 * kg);
+                unsigned char* p = at + (size_t)kg * npos * 16;
+                const auto put = [&](int d) { *reinterpret_cast<uint4*>(p + d) = w; };
+                put(0);
+                if constexpr (!IMAGES) continue;
+                if (dx) put(dx);
+                if (dy) put(dy);
+                if (dx && dy) put(dx + dy);
+                if (ND == 3 && dz) {
+                    put(dz);
+                    if (dx) put(dz + dx);
+                    if (dy) put(dz + dy);
+                    if (dx && dy) put(dz + dx + dy);
+                }
             }
         }
     }
@@ -384,8 +422,9 @@ __device__ __forceinline__ void issue_tile_c8(int first, int P, int PP, uint32_t
 // their phases), so that one half's CUDA-core phases overlap the other's
 // tensor-core phases: the runtime places a single CTA of a tcgen05 kernel
 // on an SM.
-template <int ND, int CP, bool INVERSE, int H>
-__global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs a) {
+template <int ND, int CP, bool INVERSE, int H, int NG>
+__global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const TcArgs a) {
+    constexpr int kTcThreads = tc_threads<NG>(), kTcRing = kTcRings / NG;   // accumulators per group (at most)
     constexpr int NKG = CP / 8;
     constexpr int N2 = tc_n2<CP>();
     extern __shared__ __align__(1024) unsigned char smem_all[];
@@ -400,11 +439,11 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
     FF* red = reinterpret_cast<FF*>(smem + g.off_red);
     // TMEM accumulator rings, one per epilogue group: full = the tile's MMAs
     // done (commit), empty = its accumulator drained (the group's 128 threads)
-    uint64_t* full2 = reinterpret_cast<uint64_t*>(smem + g.off_bar);   // [2][kTcRing]
-    uint64_t* empty2 = full2 + 2 * kTcRing;
-    uint64_t* full3 = empty2 + 2 * kTcRing;
-    uint64_t* empty3 = full3 + 2 * kTcRing;
-    uint64_t* done2 = empty3 + 2 * kTcRing;                              // [kTcMaxTiles]: conv2 tile done, once a layer
+    uint64_t* full2 = reinterpret_cast<uint64_t*>(smem + g.off_bar);   // [NG][kTcRing]
+    uint64_t* empty2 = full2 + kTcRings;
+    uint64_t* full3 = empty2 + kTcRings;
+    uint64_t* empty3 = full3 + kTcRings;
+    uint64_t* done2 = empty3 + kTcRings;                              // [kTcMaxTiles]: conv2 tile done, once a layer
     uint64_t* bar_w2 = done2 + kTcMaxTiles;                              // a layer's W2 staged
     uint64_t* bar_w3 = bar_w2 + 1;                                       // a layer's W3 staged
     uint64_t* bar_wf = bar_w3 + 1;                                       // 2: a layer's FP32 part staged
@@ -419,29 +458,29 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
     const int V = g.V, L = g.L, npos = g.npos, nt = g.n_tiles, P = g.P, PP = g.P * g.P, p_first = g.p_first;
     const int nb2 = g.nbuf2, nb3 = g.nbuf3, r_lag = g.r_lag;
     const FastDiv fdP = g.fd_P, fdPP = g.fd_PP;
+    // h1's periodic images by a pass of their own (as h2's) on the larger 2D
+    // lattices with 16 channels and more (2 % to 5 % faster there), else by conv1
+    const bool halo_pass = ND == 2 && CP >= 16 && L >= 32;
     const uint32_t a_ks = 2u * (uint32_t)npos;
     const int wf_floats = (int)(g.wf_bytes >> 2);
     const int64_t b0 = (int64_t)blockIdx.x * H + h, bstride = (int64_t)gridDim.x * H;
     const int64_t n_cfg = a.B > b0 ? (a.B - 1 - b0) / bstride + 1 : 0;
     const int64_t total_steps = n_cfg * a.n_layers;   // this half's layer applications
     int64_t w2_issued = -1, w3_issued = -1, wf_issued = -1;   // thread 0: the last staged steps
-    // epilogue warps: group eg (0: warps 4..7, 1: warps 8..11) takes the tiles
-    // t = eg (mod 2) through its own TMEM ring; warp w reads lane quarter w mod 4
+    // epilogue warps: group eg (warps 4 + 4 eg .. 7 + 4 eg) takes the tiles
+    // t = eg (mod NG) through its own TMEM ring; warp w reads lane quarter w mod 4
     const int eg = warp >= 4 ? (warp - 4) >> 2 : -1, q = warp & 3;
 
-    const auto block_of = [&](int64_t step) {
-        const int li = (int)(step % a.n_layers);
-        return a.Wl + (size_t)(INVERSE ? a.n_layers - 1 - li : li) * g.layer_bytes;
-    };
-    const auto stage = [&](int64_t step, void* dst, uint32_t off, uint32_t bytes, uint64_t* bar) {
+    // weights of step `step`, whose layer is number li in order of application
+    const auto stage = [&](int li, void* dst, uint32_t off, uint32_t bytes, uint64_t* bar) {
         fence_proxy_async();
         mbar_expect_tx(bar, bytes);
-        bulk_g2s(dst, block_of(step) + off, bytes, bar);
+        bulk_g2s(dst, a.Wl + (size_t)(INVERSE ? a.n_layers - 1 - li : li) * g.layer_bytes + off, bytes, bar);
     };
-    const auto stage_w2 = [&](int64_t step) { stage(step, w2s, 0, g.w2_bytes, bar_w2); w2_issued = step; };
-    const auto stage_w3 = [&](int64_t step) { stage(step, w3s, g.w2_bytes, g.w3_bytes, bar_w3); w3_issued = step; };
-    const auto stage_wf = [&](int64_t step) {
-        stage(step, wfs + (int)(step & 1) * wf_floats, g.w2_bytes + g.w3_bytes, g.wf_bytes, bar_wf + (step & 1));
+    const auto stage_w2 = [&](int64_t step, int li) { stage(li, w2s, 0, g.w2_bytes, bar_w2); w2_issued = step; };
+    const auto stage_w3 = [&](int64_t step, int li) { stage(li, w3s, g.w2_bytes, g.w3_bytes, bar_w3); w3_issued = step; };
+    const auto stage_wf = [&](int64_t step, int li) {
+        stage(li, wfs + (int)(step & 1) * wf_floats, g.w2_bytes + g.w3_bytes, g.wf_bytes, bar_wf + (step & 1));
         wf_issued = step;
     };
 
@@ -467,7 +506,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
         return ff_to_double(r);
     };
     if (tid == 0) {
-        for (int i = 0; i < 2 * kTcRing; ++i) {
+        for (int i = 0; i < kTcRings; ++i) {
             mbar_init(full2 + i, 1);
             mbar_init(empty2 + i, 4 * 32);
             mbar_init(full3 + i, 1);
@@ -478,7 +517,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
         mbar_init(bar_w3, 1);
         mbar_init(bar_wf, 1);
         mbar_init(bar_wf + 1, 1);
-        mbar_init(bar_fin, 2);                 // one commit per issuing thread
+        mbar_init(bar_fin, NG);                // one commit per issuing thread
         mbar_init(bar_stall, 1);
         *abort_flag = 0;
         fence_mbar_init();
@@ -492,9 +531,9 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
     __syncthreads();
     fence_after_sync();
     if (tid == 0 && total_steps > 0) {
-        stage_w2(0);
-        stage_w3(0);
-        stage_wf(0);
+        stage_w2(0, 0);
+        stage_w3(0, 0);
+        stage_wf(0, 0);
     }
     const uint32_t tmem = *tmem_slot0 + (uint32_t)(h * g.tmem_cols);
     // D = F32, K-major A and B, M = 128: conv2 BF16 with N = 3 CP, conv3 FP16 with N = 16
@@ -554,22 +593,36 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
 
         FF logdet{0.f, 0.f};
         for (int li = 0; li < a.n_layers; ++li, ++step) {
-            const int l = INVERSE ? a.n_layers - 1 - li : li;
+            const int l = INVERSE ? a.n_layers - 1 - li : li, next_li = li + 1 == a.n_layers ? 0 : li + 1;
             const int frozen = l & 1;
             const float* wf = wfs + (int)(step & 1) * wf_floats;
 
             // ---- conv1 -> h1 (BF16, padded, with periodic images)
             if (tc_wait(bar_wf + (step & 1), step >> 1, abort_flag, a.status)) {
-                if (tid == 0 && step + 1 < total_steps) stage_wf(step + 1);
-                tc_conv1<ND, CP, H == 1 ? 2 : 1>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+                if (tid == 0 && step + 1 < total_steps) stage_wf(step + 1, next_li);
+                // Two sites per thread share the weight loads; 16 channels per item,
+                // all 32 where one configuration's 12 warps have registers for them.
+                // A round of two sites takes about 1.6 times one of single sites.
+                constexpr int CH = CP < 16 || (H == 1 && NG == 2) ? CP : 16, NCB = CP / CH;
+                const int rounds1 = (V * NCB + kTcThreads - 1) / kTcThreads, rounds2 = (V / 2 * NCB + kTcThreads - 1) / kTcThreads;
+                if (halo_pass)
+                    tc_conv1<ND, CP, 2, CH, false>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+                else if (8 * rounds2 < 5 * rounds1)
+                    tc_conv1<ND, CP, 2, CH, true>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+                else
+                    tc_conv1<ND, CP, 1, CH, true>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+            }
+            if (halo_pass) {
+                half_sync();
+                tc_halo<ND, CP>(g, act, tid, kTcThreads);
             }
             fence_proxy_async();
             half_sync();
             if (*abort_flag) break;
 
             // ---- conv2 on the tensor cores; the epilogue writes h2 (FP16) over h1 in place
-            if (warp < 2) {
-                // issuing thread r (lane 0 of warp r, sub-partition r): tiles t = r (mod 2) into ring r
+            if (warp < NG) {
+                // issuing thread r (lane 0 of warp r, sub-partition r): tiles t = r (mod NG) into ring r
                 bool go = lane == 0;
                 if (go && a.stall_spins > 0 && step == 0 && warp == 0) {
                     // failure-path test: a wait for a completion that never comes,
@@ -584,7 +637,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
                 }
                 if (go && tc_wait(bar_w2, step, abort_flag, a.status)) {
                     fence_after_sync();
-                    for (int t = warp; t < nt; t += 2) {
+                    for (int t = warp; t < nt; t += NG) {
                         if (k2 >= 1) {
                             if (!tc_wait(empty2 + warp * kTcRing + i2, k2 - 1, abort_flag, a.status)) break;
                             fence_after_sync();
@@ -603,45 +656,73 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
                 __syncwarp();
             } else if (eg >= 0) {
                 const float* b2 = wf + g.wf_b2;
+                const f32x2 slope2 = f2_splat(a.slope);
                 int dwaited = 0;           // tiles whose completion this thread has seen (done2)
                 bool ok = true;
-                for (int t = eg; t < nt && ok; t += 2) {
+                for (int t = eg; t < nt && ok; t += NG) {
                     if (!(ok = tc_wait(full2 + eg * kTcRing + i2, k2, abort_flag, a.status))) break;
                     fence_after_sync();
                     // out = D_0(left) + D_1 + D_2(right) + b2, 16 channels at a time, LeakyReLU
                     const uint32_t tcol = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((eg * nb2 + i2) * N2);
-                    float out[CP];
+                    uint4 out[NKG];
                     if constexpr (CP == 8) {
                         // columns dx 8 + c; 24..31 are the zero padding of N
-                        float v01[16], v2p[16];
+                        float v01[16], v2p[16], o[8];
+                        f32x2 b[4], sum[4];
                         tmem_ld16(tcol, v01);
                         tmem_ld16(tcol + 16, v2p);
+                        load_pairs<8>(b, b2);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            const float left = __shfl_up_sync(0xffffffffu, v01[c], 1, 8);
-                            const float right = __shfl_down_sync(0xffffffffu, v2p[c], 1, 8);
-                            out[c] = lrelu_tc(left + v01[8 + c] + right + b2[c], a.slope);
+                        for (int c = 0; c < 4; ++c) {
+                            const f32x2 left = f2_make(__shfl_up_sync(0xffffffffu, v01[2 * c], 1, 8),
+                                                       __shfl_up_sync(0xffffffffu, v01[2 * c + 1], 1, 8));
+                            const f32x2 right = f2_make(__shfl_down_sync(0xffffffffu, v2p[2 * c], 1, 8),
+                                                        __shfl_down_sync(0xffffffffu, v2p[2 * c + 1], 1, 8));
+                            sum[c] = f2_add(f2_add(f2_add(left, f2_make(v01[8 + 2 * c], v01[9 + 2 * c])), right), b[c]);
                         }
+                        lrelu_pairs(sum, slope2, o);
+                        out[0] = pack_f16x8(o);
                     }
 #pragma unroll
                     for (int h = 0; h < CP / 16; ++h) {
-                        float v0[16], v1[16], v2[16];
+                        // (packed arithmetic where two configurations share the issue slots;
+                        // with one, the scalar form's shorter chains are 1 % to 4 % faster)
+                        float v0[16], v1[16], v2[16], o[16];
                         tmem_ld16(tcol + h * 16, v0);
                         tmem_ld16(tcol + CP + h * 16, v1);
                         tmem_ld16(tcol + 2 * CP + h * 16, v2);
-                        tmem_ld_wait();
+                        if constexpr (H == 2) {
+                            f32x2 b[8], sum[8];
+                            load_pairs<16>(b, b2 + h * 16);
+                            tmem_ld_wait();
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const float left = __shfl_up_sync(0xffffffffu, v0[c], 1, 8);
-                            const float right = __shfl_down_sync(0xffffffffu, v2[c], 1, 8);
-                            out[h * 16 + c] = lrelu_tc(left + v1[c] + right + b2[h * 16 + c], a.slope);
+                            for (int c = 0; c < 8; ++c) {
+                                const f32x2 left = f2_make(__shfl_up_sync(0xffffffffu, v0[2 * c], 1, 8),
+                                                           __shfl_up_sync(0xffffffffu, v0[2 * c + 1], 1, 8));
+                                const f32x2 right = f2_make(__shfl_down_sync(0xffffffffu, v2[2 * c], 1, 8),
+                                                            __shfl_down_sync(0xffffffffu, v2[2 * c + 1], 1, 8));
+                                sum[c] = f2_add(f2_add(f2_add(left, f2_make(v1[2 * c], v1[2 * c + 1])), right), b[c]);
+                            }
+                            lrelu_pairs(sum, slope2, o);
+                        } else {
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) {
+                                const float left = __shfl_up_sync(0xffffffffu, v0[c], 1, 8);
+                                const float right = __shfl_down_sync(0xffffffffu, v2[c], 1, 8);
+                                const float sum = left + v1[c] + right + b2[h * 16 + c];
+                                o[c] = sum > 0.f ? sum : a.slope * sum;
+                            }
                         }
+                        out[2 * h] = pack_f16x8(o);
+                        out[2 * h + 1] = pack_f16x8(o + 8);
                     }
                     fence_before_sync();
                     mbar_arrive(empty2 + eg * kTcRing + i2);
                     if (++i2 == nb2) { i2 = 0; ++k2; }
-                    // h2 of tile t may overwrite h1 once tiles t .. t + r_lag are done
+                    // h2 of tile t may overwrite h1 once tiles t .. t + r_lag are done (holding
+                    // it back until after the next tile's arithmetic was 10 % to 20 % slower)
                     const int need = t + r_lag < nt ? t + r_lag : nt - 1;
                     while (ok && dwaited <= need) {
                         ok = tc_wait(done2 + dwaited, step, abort_flag, a.status);
@@ -654,7 +735,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
                     if (rvalid && px >= 1 && px <= L && py >= 1 && py <= L && pz >= 1 && pz <= L) {
 #pragma unroll
                         for (int kg = 0; kg < NKG; ++kg)
-                            *reinterpret_cast<uint4*>(act + ((size_t)kg * npos + p) * 16) = pack_f16x8(out + kg * 8);
+                            *reinterpret_cast<uint4*>(act + ((size_t)kg * npos + p) * 16) = out[kg];
                     }
                 }
             }
@@ -663,7 +744,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
             if (*abort_flag) break;
             fence_after_sync();
             // every conv2 MMA of this layer has completed: the next layer's W2 may land
-            if (tid == 0 && step + 1 < total_steps) stage_w2(step + 1);
+            if (tid == 0 && step + 1 < total_steps) stage_w2(step + 1, next_li);
 
             // ---- periodic images of h2
             tc_halo<ND, CP>(g, act, tid, kTcThreads);
@@ -671,10 +752,10 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
             half_sync();
 
             // ---- conv3 (s, t) on the tensor cores; the epilogue updates the other parity
-            if (warp < 2) {
+            if (warp < NG) {
                 if (lane == 0 && tc_wait(bar_w3, step, abort_flag, a.status)) {
                     fence_after_sync();
-                    for (int t = warp; t < nt; t += 2) {
+                    for (int t = warp; t < nt; t += NG) {
                         if (k3 >= 1) {
                             if (!tc_wait(empty3 + warp * kTcRing + i3, k3 - 1, abort_flag, a.status)) break;
                             fence_after_sync();
@@ -694,7 +775,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
                 const float bs = wf[g.wf_b3], bt = wf[g.wf_b3 + 1];
                 const int pa = frozen ^ 1;
                 bool ok = true;
-                for (int t = eg; t < nt && ok; t += 2) {
+                for (int t = eg; t < nt && ok; t += NG) {
                     if (!(ok = tc_wait(full3 + eg * kTcRing + i3, k3, abort_flag, a.status))) break;
                     fence_after_sync();
                     float v[8];
@@ -730,7 +811,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
             if (*abort_flag) break;
             fence_after_sync();
             // every conv3 MMA of this layer has completed: the next layer's W3 may land
-            if (tid == 0 && step + 1 < total_steps) stage_w3(step + 1);
+            if (tid == 0 && step + 1 < total_steps) stage_w3(step + 1, next_li);
         }
         if (*abort_flag) break;
 
@@ -761,7 +842,7 @@ __global__ void __launch_bounds__(kTcThreads * H, 1) flow_tc_kernel(const TcArgs
     }
     // teardown: copies still landing and MMAs still queued (only after an
     // abort) finish before their shared memory and TMEM are released
-    if (warp < 2 && lane == 0) mma_commit(bar_fin);
+    if (warp < NG && lane == 0) mma_commit(bar_fin);
     if (tid == 0) {
         if (w2_issued >= 0) tc_drain(bar_w2, w2_issued);
         if (w3_issued >= 0) tc_drain(bar_w3, w3_issued);
@@ -898,14 +979,15 @@ bool tc_plan(const gf_flow_shape& s, TcGeom& g) {
     g.off_x = g.off_wf + 2 * g.wf_bytes;
     g.off_red = g.off_x + (uint32_t)((g.V * 4 + 15) & ~15);
     g.off_bar = g.off_red + 32 * 8;
-    g.smem_need = g.off_bar + (8 * kTcRing + kTcMaxTiles + 6) * 8 + 16;
+    g.smem_need = g.off_bar + (4 * kTcRings + kTcMaxTiles + 6) * 8 + 16;
     g.half_bytes = (g.smem_need + 1023) & ~1023u;
     return g.smem_need <= (uint32_t)kSmemPerCTA;
 }
 
-template <int ND, int CP, bool INV, int H>
+template <int ND, int CP, bool INV, int H, int NG>
 gf_status launch_tc(TcArgs& a, cudaStream_t stream) {
-    auto kern = flow_tc_kernel<ND, CP, INV, H>;
+    constexpr int kTcThreads = tc_threads<NG>(), kTcRing = kTcRings / NG;
+    auto kern = flow_tc_kernel<ND, CP, INV, H, NG>;
     TcGeom& g = a.g;
     const size_t smem = (size_t)H * g.half_bytes;
     if (smem > (size_t)kSmemPerCTA) return GF_EUNSUPPORTED;
@@ -932,15 +1014,16 @@ gf_status launch_tc(TcArgs& a, cudaStream_t stream) {
         if (checked[dev] < 0) return GF_EUNSUPPORTED;
     }
     g.tmem_cols = 512 / H;
-    g.nbuf2 = std::min(kTcRing, g.tmem_cols / (2 * tc_n2<CP>()));
-    g.nbuf3 = std::min(kTcRing, g.tmem_cols / (2 * 16));
+    g.nbuf2 = std::min(kTcRing, g.tmem_cols / (NG * tc_n2<CP>()));
+    g.nbuf3 = std::min(kTcRing, g.tmem_cols / (NG * 16));
     if (g.nbuf2 < 1 || g.nbuf3 < 1) return GF_EUNSUPPORTED;
-    // the conv2 schedule needs r_lag <= 2 nbuf2 (+ 1 when r_lag is odd): an
-    // epilogue group holding tile t's store waits for tile t + r_lag's MMAs,
-    // whose accumulator is the one tile t + r_lag - 2 nbuf2 used, drained only
-    // by a group that has reached that tile (the same group when r_lag is
-    // even, which has drained up to t; the other, up to t + 1, when odd)
-    if (g.r_lag > 2 * g.nbuf2 + (g.r_lag & 1)) return GF_EUNSUPPORTED;
+    // the conv2 schedule needs r_lag <= NG nbuf2 + (r_lag mod NG): an epilogue
+    // group holding tile t's store waits for tile t + r_lag's MMAs, whose
+    // accumulator is the one tile t + r_lag - NG nbuf2 used, drained by a group
+    // that has reached that tile; with t the earliest tile held, that group has
+    // reached (and drained before waiting) its first tile from t on, tile
+    // t + (r_lag mod NG)
+    if (g.r_lag > NG * g.nbuf2 + g.r_lag % NG) return GF_EUNSUPPORTED;
     const int64_t grid = std::min<int64_t>((a.B + H - 1) / H, (int64_t)num_sms());
     if (grid <= 0) return GF_OK;
     kern<<<(unsigned)grid, kTcThreads * H, smem, stream>>>(a);
@@ -998,29 +1081,24 @@ gf_status launch_flow_tc(const gf_flow* f, bool inverse, const gf_phi4* phi4, in
     a.status = status_word(stream);
     a.stall_spins = bf16_stall_spins();
     if (!a.status) return GF_ECUDA;
-    const bool c32 = a.g.Cp == 32, c8 = a.g.Cp == 8;
-    // two configurations per CTA where two halves' shared memory fits (every
-    // 2D lattice but the largest; 3D L = 8 with widths 8, 16 and L = 12 with 8)
-    const bool two = 2 * (size_t)a.g.half_bytes <= (size_t)kSmemPerCTA && B > num_sms();
-    if (f->shape.nd == 3) {
-        if (c32) return inverse ? launch_tc<3, 32, true, 1>(a, stream) : launch_tc<3, 32, false, 1>(a, stream);
-        if (c8) {
-            if (two) return inverse ? launch_tc<3, 8, true, 2>(a, stream) : launch_tc<3, 8, false, 2>(a, stream);
-            return inverse ? launch_tc<3, 8, true, 1>(a, stream) : launch_tc<3, 8, false, 1>(a, stream);
-        }
-        if (two) return inverse ? launch_tc<3, 16, true, 2>(a, stream) : launch_tc<3, 16, false, 2>(a, stream);
-        return inverse ? launch_tc<3, 16, true, 1>(a, stream) : launch_tc<3, 16, false, 1>(a, stream);
-    }
-    if (c8) {
-        if (two) return inverse ? launch_tc<2, 8, true, 2>(a, stream) : launch_tc<2, 8, false, 2>(a, stream);
-        return inverse ? launch_tc<2, 8, true, 1>(a, stream) : launch_tc<2, 8, false, 1>(a, stream);
-    }
-    if (c32) {
-        if (two) return inverse ? launch_tc<2, 32, true, 2>(a, stream) : launch_tc<2, 32, false, 2>(a, stream);
-        return inverse ? launch_tc<2, 32, true, 1>(a, stream) : launch_tc<2, 32, false, 1>(a, stream);
-    }
-    if (two) return inverse ? launch_tc<2, 16, true, 2>(a, stream) : launch_tc<2, 16, false, 2>(a, stream);
-    return inverse ? launch_tc<2, 16, true, 1>(a, stream) : launch_tc<2, 16, false, 1>(a, stream);
+    // Two configurations per CTA where two halves' shared memory fits (every 2D
+    // lattice but the largest; 3D L = 8 with widths 8, 16 and L = 12 with 8) and
+    // the batch fills more than one per SM; where two never fit, one with four
+    // epilogue groups.
+    const bool fits = 2 * (size_t)a.g.half_bytes <= (size_t)kSmemPerCTA, two = fits && B > num_sms();
+    const auto go = [&](auto nd, auto cp) -> gf_status {
+        constexpr int ND = decltype(nd)::value, CP = decltype(cp)::value;
+        if (two) return inverse ? launch_tc<ND, CP, true, 2, 2>(a, stream) : launch_tc<ND, CP, false, 2, 2>(a, stream);
+        if (fits) return inverse ? launch_tc<ND, CP, true, 1, 2>(a, stream) : launch_tc<ND, CP, false, 1, 2>(a, stream);
+        constexpr int NG = CP == 32 ? 2 : 4;      // (width 32: four groups would have one accumulator each)
+        return inverse ? launch_tc<ND, CP, true, 1, NG>(a, stream) : launch_tc<ND, CP, false, 1, NG>(a, stream);
+    };
+    const auto width = [&](auto nd) -> gf_status {
+        if (a.g.Cp == 32) return go(nd, std::integral_constant<int, 32>());
+        if (a.g.Cp == 16) return go(nd, std::integral_constant<int, 16>());
+        return go(nd, std::integral_constant<int, 8>());
+    };
+    return f->shape.nd == 3 ? width(std::integral_constant<int, 3>()) : width(std::integral_constant<int, 2>());
 }
 
 }  // namespace gf
