@@ -458,9 +458,12 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
     const int V = g.V, L = g.L, npos = g.npos, nt = g.n_tiles, P = g.P, PP = g.P * g.P, p_first = g.p_first;
     const int nb2 = g.nbuf2, nb3 = g.nbuf3, r_lag = g.r_lag;
     const FastDiv fdP = g.fd_P, fdPP = g.fd_PP;
-    // h1's periodic images by a pass of their own (as h2's) on the larger 2D
-    // lattices with 16 channels and more (2 % to 5 % faster there), else by conv1
-    const bool halo_pass = ND == 2 && CP >= 16 && L >= 32;
+    // h1's periodic images by a pass of their own (as h2's) on 2D lattices from
+    // L = 16 with 16 channels and from L = 32 with 32, else by conv1 (3000
+    // configurations, 16 layers, by conv1 -> by a pass, us: hidden 16 L = 8
+    // 671 -> 907, L = 16 987 -> 955, L = 24 1635 -> 1587, L = 64 (1500) 4058 ->
+    // 3947; hidden 32 L = 16 1364 -> 1377, L = 48 (2000) 5438 -> 5377)
+    const bool halo_pass = ND == 2 && CP >= 16 && L >= CP;
     const uint32_t a_ks = 2u * (uint32_t)npos;
     const int wf_floats = (int)(g.wf_bytes >> 2);
     const int64_t b0 = (int64_t)blockIdx.x * H + h, bstride = (int64_t)gridDim.x * H;
@@ -602,15 +605,20 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                 if (tid == 0 && step + 1 < total_steps) stage_wf(step + 1, next_li);
                 // Two sites per thread share the weight loads; 16 channels per item,
                 // all 32 where one configuration's 12 warps have registers for them.
-                // A round of two sites takes about 1.6 times one of single sites.
+                // A round of two sites takes about 1.6 times one of single sites in 3D
+                // (27 taps) and twice in 2D, where pairs gain with 32 channels alone
+                // (2D L = 24, hidden 16, 3000 configurations: single 1587 us, pairs 1685).
                 constexpr int CH = CP < 16 || (H == 1 && NG == 2) ? CP : 16, NCB = CP / CH;
                 const int rounds1 = (V * NCB + kTcThreads - 1) / kTcThreads, rounds2 = (V / 2 * NCB + kTcThreads - 1) / kTcThreads;
-                if (halo_pass)
-                    tc_conv1<ND, CP, 2, CH, false>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
-                else if (8 * rounds2 < 5 * rounds1)
+                const bool pairs = ND == 3 ? 8 * rounds2 < 5 * rounds1 : CP == 32 && 2 * rounds2 <= rounds1;
+                if (halo_pass) {
+                    if constexpr (ND == 2 && CP >= 16)
+                        tc_conv1<ND, CP, CP / 16, CH, false>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+                } else if (pairs) {
                     tc_conv1<ND, CP, 2, CH, true>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
-                else
+                } else {
                     tc_conv1<ND, CP, 1, CH, true>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
+                }
             }
             if (halo_pass) {
                 half_sync();
