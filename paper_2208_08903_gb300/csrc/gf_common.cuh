@@ -238,7 +238,7 @@ __device__ __forceinline__ double lap_minus(const T* p, int n, int nd, int L) {
 
 // The force dS/dphi(n) = 2 sum_mu (2 phi - phi(n+mu) - phi(n-mu)) + 2 m2 phi
 // + 4 lam phi^3 in FP64: the one definition used by gf_phi4_force, the action
-// VJP, the HMC kicks and the training reverse pass's seed.
+// VJP and the training reverse pass's seed; the HMC kicks use the form below.
 template <typename T>
 __device__ __forceinline__ double phi4_force_at(const T* p, int n, int nd, const SiteNbrs& b, double m2, double lam) {
     const double c = (double)p[n];
@@ -247,6 +247,17 @@ __device__ __forceinline__ double phi4_force_at(const T* p, int n, int nd, const
 template <typename T>
 __device__ __forceinline__ double phi4_force_site(const T* p, int n, int nd, int L, double m2, double lam) {
     return phi4_force_at(p, n, nd, site_nbrs(n, nd, L), m2, lam);
+}
+
+// The same force for a kick of step h, folded into three coefficients (fewer
+// FP64 instructions): momentum - h dS/dphi at a site of value f (f2 = f^2) whose
+// neighbours sum to s.
+struct Phi4Kick { double k1, k3, kn; };
+__device__ __forceinline__ Phi4Kick phi4_kick(double h, int nd, double m2, double lam) {
+    return {-2.0 * h * (2 * nd + m2), -4.0 * h * lam, 2.0 * h};
+}
+__device__ __forceinline__ double phi4_force_at(const Phi4Kick& k, double f, double f2, double s, double momentum) {
+    return fma(k.kn, s, fma(fma(k.k3, f2, k.k1), f, momentum));
 }
 
 // phi^4 action (paper Sec. 1) of one configuration held in shared memory,

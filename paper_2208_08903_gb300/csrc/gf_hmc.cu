@@ -76,7 +76,8 @@ __global__ void __launch_bounds__(kHmcThreads, 2) hmc_kernel(int L, int lg, int 
         // H = sum 1/2 pi^2 + (2 nd + m2) phi^2 + lam phi^4 - phi (sum of neighbours)
         const auto kick = [&](double h, auto with_energy) -> double {
             constexpr int E = decltype(with_energy)::value;
-            const double k1 = -2.0 * h * (2 * ND + m2), k3 = -4.0 * h * lam, kn = 2.0 * h, c2 = 2 * ND + m2;
+            const Phi4Kick kk = phi4_kick(h, ND, m2, lam);
+            const double c2 = 2 * ND + m2;
             double kin = 0.0, pot = 0.0, hop = 0.0;
 #pragma unroll
             for (int k = 0; k < kMaxSitesPerThread; ++k) {
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(kHmcThreads, 2) hmc_kernel(int L, int lg, int 
                     double s = (p[b.xp] + p[b.xm]) + (p[b.yp] + p[b.ym]);
                     if (ND == 3) s += p[b.zp] + p[b.zm];
                     if (E < 0) kin = fma(pi[k], pi[k], kin);
-                    pi[k] = fma(kn, s, fma(fma(k3, f2, k1), f, pi[k]));
+                    pi[k] = phi4_force_at(kk, f, f2, s, pi[k]);
                     if (E > 0) kin = fma(pi[k], pi[k], kin);
                     if (E != 0) {
                         pot = fma(f2, fma(lam, f2, c2), pot);
