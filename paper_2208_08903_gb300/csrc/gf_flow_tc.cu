@@ -605,12 +605,13 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                 if (tid == 0 && step + 1 < total_steps) stage_wf(step + 1, next_li);
                 // Two sites per thread share the weight loads; 16 channels per item,
                 // all 32 where one configuration's 12 warps have registers for them.
-                // A round of two sites takes about 1.6 times one of single sites in 3D
-                // (27 taps) and twice in 2D, where pairs gain with 32 channels alone
-                // (2D L = 24, hidden 16, 3000 configurations: single 1587 us, pairs 1685).
+                // A round of pairs must stand for two of single sites, and in 2D pairs gain
+                // with 32 channels alone (single -> pairs, us: 3D L = 8, hidden 8, 3000
+                // configurations, rounds 2 -> 1, 1902 -> 1827; 3D L = 12, hidden 8, 458,
+                // rounds 5 -> 3, 985 -> 1024; 2D L = 24, hidden 16, 3000 1587 -> 1685).
                 constexpr int CH = CP < 16 || (H == 1 && NG == 2) ? CP : 16, NCB = CP / CH;
                 const int rounds1 = (V * NCB + kTcThreads - 1) / kTcThreads, rounds2 = (V / 2 * NCB + kTcThreads - 1) / kTcThreads;
-                const bool pairs = ND == 3 ? 8 * rounds2 < 5 * rounds1 : CP == 32 && 2 * rounds2 <= rounds1;
+                const bool pairs = (ND == 3 || CP == 32) && 2 * rounds2 <= rounds1;
                 if (halo_pass) {
                     if constexpr (ND == 2 && CP >= 16)
                         tc_conv1<ND, CP, CP / 16, CH, false>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
