@@ -24,8 +24,8 @@
 // (registers, or the buffers' shared memory, allow 16 to 24 an SM).  One site per
 // thread with the weights through L1 was bound by load issue (8 FMAs to 3 loads)
 // and waited for L2 at the start of every convolution: 2D L = 16, 12 layers,
-// widths 16, 16, 8, 5 taps, 500 configurations 2980 us, now 1311 (23 TFLOP/s);
-// 3D L = 8, widths 16, 8, 16, 4 layers, 300 configurations 1279 -> 425.
+// widths 16, 16, 8, 5 taps, 500 configurations 3004 us, now 1319 (23 TFLOP/s);
+// 3D L = 8, widths 16, 8, 16, 4 layers, 300 configurations 1291 -> 419.
 //
 // Each sum runs over taps, then input channels, from the bias, and the lattice
 // sums are added as by `vthreads` threads whatever the CTA's size, so results
@@ -138,7 +138,7 @@ struct Walk { int kx, ky, kz, ci; };
 // inputs.  Site s is at (xc[s], y[s], z[s]), or all at xc[0] (NX = 1); its row of `stride` floats starts at
 // in + site * stride.  zero >= 0: a masked input (one channel), read at the
 // sites of parity `frozen` and as the zero at smv[zero] elsewhere.
-template <int ND, int NS, int NX, int CO, bool STAGED>
+template <int ND, int NS, int NX, int CO, bool STAGED, bool ONE>
 __device__ __forceinline__ void add_rows(const VarArgs& a, f32x2 (&acc)[NS][CO / 2], Walk& w, const int (&xc)[NX], const int (&y)[NS],
                                          const int (&z)[NS], const float* wg, int ws, int cop, int rows, int cin, int in,
                                          int stride, int zero, int frozen) {
@@ -161,11 +161,11 @@ __device__ __forceinline__ void add_rows(const VarArgs& a, f32x2 (&acc)[NS][CO /
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
             const int X = xx[NX == 1 ? 0 : s];
-            q[s] = at[s] + X * stride + w.ci;
-            if (zero >= 0 && ((X + odd[s]) & 1)) q[s] = zero;
+            q[s] = ONE ? at[s] + X * stride : at[s] + X * stride + w.ci;
+            if (ONE && zero >= 0 && ((X + odd[s]) & 1)) q[s] = zero;
         }
-        const int e = min(cin - w.ci, rows);
-#pragma unroll 4
+        const int e = ONE ? 1 : min(cin - w.ci, rows);
+#pragma unroll (ONE ? 1 : 4)
         for (int i = 0; i < e; ++i) {
             f32x2 wv[CO / 2], v[NS];
             if constexpr (CO == 2) {
@@ -189,8 +189,8 @@ __device__ __forceinline__ void add_rows(const VarArgs& a, f32x2 (&acc)[NS][CO /
             else wg += cop;
         }
         rows -= e;
-        w.ci += e;
-        if (w.ci == cin) {
+        if (!ONE) w.ci += e;
+        if (ONE || w.ci == cin) {
             w.ci = 0;
             if (++w.kx == K) {
                 w.kx = 0;
@@ -241,12 +241,18 @@ __device__ void hidden_conv(const VarArgs& a, Stream& st, const float* __restric
             }
             const float* wg = Wl + a.woff[j] + (size_t)r0 * cop + co;
             if (eight) {
-                add_rows<ND, NS, 1, 8, STAGED>(a, acc, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
+                if (cin == 1)
+                    add_rows<ND, NS, 1, 8, STAGED, true>(a, acc, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
+                else
+                    add_rows<ND, NS, 1, 8, STAGED, false>(a, acc, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
             } else {
                 f32x2 four[NS][2];
 #pragma unroll
                 for (int s = 0; s < NS; ++s) { four[s][0] = acc[s][0]; four[s][1] = acc[s][1]; }
-                add_rows<ND, NS, 1, 4, STAGED>(a, four, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
+                if (cin == 1)
+                    add_rows<ND, NS, 1, 4, STAGED, true>(a, four, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
+                else
+                    add_rows<ND, NS, 1, 4, STAGED, false>(a, four, w, xc, y, z, wg, ws + co, cop, n, cin, in, stride, zero, frozen);
 #pragma unroll
                 for (int s = 0; s < NS; ++s) { acc[s][0] = four[s][0]; acc[s][1] = four[s][1]; }
             }
@@ -306,8 +312,12 @@ __device__ void head_conv(const VarArgs& a, Stream& st, const float* __restrict_
 #pragma unroll
                     for (int s = 0; s < NS; ++s) acc[s][0] = b;
                 }
-                add_rows<ND, NS, NS, 2, STAGED>(a, acc, w, xc, y, z, Wl + a.woff[j] + (size_t)r0 * 4, ws, 4,
-                                                min(chunk, total - r0), cin, in, stride, zero, frozen);
+                const float* wg = Wl + a.woff[j] + (size_t)r0 * 4;
+                const int n = min(chunk, total - r0);
+                if (cin == 1)
+                    add_rows<ND, NS, NS, 2, STAGED, true>(a, acc, w, xc, y, z, wg, ws, 4, n, cin, in, stride, zero, frozen);
+                else
+                    add_rows<ND, NS, NS, 2, STAGED, false>(a, acc, w, xc, y, z, wg, ws, 4, n, cin, in, stride, zero, frozen);
             }
             if (!act) continue;
 #pragma unroll
@@ -612,12 +622,13 @@ gf_status launch_flow_variant(const gf_flow* f, bool inverse, const gf_phi4* phi
     }
     // CTA size and sites per thread (at most 4 with 128 registers to a thread, 2
     // with 80): those that finish the batch soonest, estimated in cycles of a
-    // layer on an SM of r CTAs as issue time (a row, one input channel of one tap,
-    // takes a warp 4 + 7 ns slots, or 8 ns cycles of its scheduler's FMA pipe) plus
-    // what one CTA alone takes (its warps in turn, 24 cycles a row per pass, 400
-    // for every barrier).  Fitted to 18 networks at 37 to 1500 configurations: the
-    // pick is within 5 % of the best but for three (2D L = 16, widths 16, 16, 8, 5
-    // taps: 256 threads 1890 us, 128 threads 1311, 64 threads 1689 for 500).
+    // layer on an SM of r CTAs as what one CTA alone takes (a row, one input channel
+    // of one tap, takes a warp 4 + 7 ns issue slots or 8 ns cycles of its
+    // scheduler's FMA pipe; a pass no less than its latencies, 24 cycles a row and 60
+    // a tap; 400 for every barrier) plus the others' issue time.  Fitted to 27
+    // networks at 37 to 8000 configurations: the pick is mostly within 5 % of the
+    // best, at worst 12 % (2D L = 16, widths 16, 16, 8, 5 taps: 256 threads 1820 us,
+    // 128 threads 1310, 64 threads 1690 for 500).
     const int64_t sms = num_sms(), by_smem = (int64_t)(228 * 1024 / (smem + 1024));
     double best = 0;
     int threads = 0, nsmax = 0, per_sm = 1;
@@ -639,11 +650,12 @@ gf_status launch_flow_variant(const gf_flow* f, bool inverse, const gf_phi4* phi
                 const double c = head ? 4.0 + 4.0 * ns[j] : std::max(8.0 * ns[j], 4.0 + 7.0 * ns[j]);
                 const double tap = f->T * (20.0 + 5.0 * ns[j]);
                 eff += tasks / 4.0 * (c * total + tap);
+                const double issue = (c + 3.0 * ns[j]) * total + tap, stall = 24.0 * total + 60.0 * f->T;
                 for (int left = tasks; left > 0; left -= warps)
-                    lat += ((std::min(left, warps) + 3) / 4) * ((c + 3.0 * ns[j]) * total + tap) + 24.0 * total +
+                    lat += std::max((std::min(left, warps) + 3) / 4 * issue, issue + stall) +
                            400.0 * (total + a.rows[j] - 1) / a.rows[j];
             }
-            const double cost = (double)((B + sms * r - 1) / (sms * r)) * (lat + r * eff);
+            const double cost = (double)((B + sms * r - 1) / (sms * r)) * (lat + (r - 0.5) * eff);
             if (threads && cost >= best) continue;
             best = cost; threads = nt; nsmax = most; per_sm = (int)fit;
             std::copy(ns, ns + f->n_hidden + 1, a.ns);
