@@ -60,6 +60,15 @@
 // on an mbarrier is bounded: a wait that runs out records GF_ETIMEOUT, raises
 // the CTA's abort flag, and the CTA leaves after draining its queued MMAs and
 // copies.
+//
+// What bounds it: chains of waits within a configuration, not the tensor pipe
+// (15 % busy).  2D L = 32, hidden 32, two configurations per CTA, cycles per
+// layer: conv1 11 K, conv2 20 K, halo 0.5 K, head 8 K.  Packed FP32 pairs in
+// conv1 and the epilogue, conv1's images as predicated stores or a pass of
+// their own, and four groups where one configuration fills the SM took, in us:
+// 2D L = 32, hidden 32, 24 layers, 8192 configurations 13436 -> 12892; 2D
+// L = 64, hidden 16, 16 layers, density of 1500 4604 -> 3853; 3D L = 12, hidden
+// 16, 16 layers, 999 configurations 2981 -> 2559.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
