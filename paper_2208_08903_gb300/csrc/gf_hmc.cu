@@ -9,13 +9,15 @@
 // The FP64 pipe bounds it: a warp's FP64 instruction takes about 19 cycles of
 // an SM (1.057 TFLOP/s on the chip), so what counts is FP64 instructions, of any
 // kind.  A site's kick is 2 nd - 1 additions of its neighbours, phi^2, and three
-// multiply-adds (with the step size folded into the coefficients), its drift
-// one: 10 in 3D.  The energies ride on the first and the last kick, whose
-// neighbour sums they share (4 more).  Each FP64 Box-Muller block (about 150
+// multiply-adds, its drift one: 10 in 3D.  The energies ride on the first and the
+// last kick: the hopping part as the squares of the nd forward differences (each
+// exact or nearly so, all of one sign), 2 nd + 3 instructions more.  From the
+// neighbour sums, in 4, two sums far larger than their difference cancelled: dH
+// of a smooth field of size 50 lost two digits.  Each FP64 Box-Muller block (about 150
 // instructions) is evaluated once, by one lane of the four whose sites it
 // serves, and exchanged by shuffles.  Measured, 20 steps, against the form with
 // the Laplacian, force and energies written out (18 FP64 instructions a step)
-// and four lanes evaluating every block: 512 chains of 3D L=16 2.39 -> 1.14 ms,
+// and four lanes evaluating every block: 512 chains of 3D L=16 2.39 -> 1.18 ms,
 // 152 chains 0.60 -> 0.30 ms, 400 chains of 2D L=64 1.58 -> 0.71 ms.  What is
 // left above the instruction count is the SMs that hold 4 of the 512 chains
 // while others hold 3.
@@ -41,7 +43,7 @@ __global__ void __launch_bounds__(kHmcThreads, 2) hmc_kernel(int L, int lg, int 
     const auto nbrs = [&](int n) { return POW2 ? site_nbrs_pow2(n, ND, lg) : site_nbrs(n, ND, L); };
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* p = reinterpret_cast<double*>(smem_raw);
-    double* red = p + V;                        // 8 warps' sums, then the chain's dH and -log u
+    double* red = p + V;                        // 8 warps' sums of H before, 8 after, then the accept flag
     const int tid = threadIdx.x, lane = tid & 31;
     const int nper = (V + kHmcThreads - 1) / kHmcThreads;
     for (int64_t c = blockIdx.x; c < n_chains; c += gridDim.x) {
@@ -73,12 +75,11 @@ __global__ void __launch_bounds__(kHmcThreads, 2) hmc_kernel(int L, int lg, int 
         __syncthreads();
         // pi -= h dS/dphi = h (2 (2 nd + m2) phi - 2 sum of neighbours + 4 lam phi^3);
         // E = -1: returns this thread's part of H before the kick, E = 1: after it.
-        // H = sum 1/2 pi^2 + (2 nd + m2) phi^2 + lam phi^4 - phi (sum of neighbours)
+        // H = sum 1/2 pi^2 + sum over mu (phi - phi(n+mu))^2 + m2 phi^2 + lam phi^4
         const auto kick = [&](double h, auto with_energy) -> double {
             constexpr int E = decltype(with_energy)::value;
             const Phi4Kick kk = phi4_kick(h, ND, m2, lam);
-            const double c2 = 2 * ND + m2;
-            double kin = 0.0, pot = 0.0, hop = 0.0;
+            double kin = 0.0, pot = 0.0;
 #pragma unroll
             for (int k = 0; k < kMaxSitesPerThread; ++k) {
                 const int n = tid + k * kHmcThreads;
@@ -91,12 +92,14 @@ __global__ void __launch_bounds__(kHmcThreads, 2) hmc_kernel(int L, int lg, int 
                     pi[k] = phi4_force_at(kk, f, f2, s, pi[k]);
                     if (E > 0) kin = fma(pi[k], pi[k], kin);
                     if (E != 0) {
-                        pot = fma(f2, fma(lam, f2, c2), pot);
-                        hop = fma(f, s, hop);
+                        const double dx = f - p[b.xp], dy = f - p[b.yp], dz = ND == 3 ? f - p[b.zp] : 0.0;
+                        pot = fma(dy, dy, fma(dx, dx, pot));
+                        if (ND == 3) pot = fma(dz, dz, pot);
+                        pot = fma(f2, fma(lam, f2, m2), pot);
                     }
                 }
             }
-            return E != 0 ? 0.5 * kin + (pot - hop) : 0.0;
+            return E != 0 ? fma(0.5, kin, pot) : 0.0;
         };
         const double h0 = kick(0.5 * eps, std::integral_constant<int, -1>());
         double h1 = 0.0;
