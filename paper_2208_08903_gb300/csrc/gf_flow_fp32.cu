@@ -113,17 +113,17 @@ bool set_h2(gf_flow* f, const std::vector<Phase>& s) {
     return true;
 }
 
-FlowKernel kernel_for(const gf_flow* f, int tile, bool rec) {
+FlowKernel kernel_for(const gf_flow* f, int tile, int mode) {
     const bool gw = f->weights_global;
     switch (f->shape.nd * 100 + f->C1) {
-        case 208: return kernel_of<2, 8>(tile, gw, rec);
-        case 216: return kernel_of<2, 16>(tile, gw, rec);
-        case 224: return kernel_of<2, 24>(tile, gw, rec);
-        case 232: return kernel_of<2, 32>(tile, gw, rec);
-        case 308: return kernel_of<3, 8>(tile, gw, rec);
-        case 316: return kernel_of<3, 16>(tile, gw, rec);
-        case 324: return kernel_of<3, 24>(tile, gw, rec);
-        default: return kernel_of<3, 32>(tile, gw, rec);
+        case 208: return kernel_of<2, 8>(tile, gw, mode);
+        case 216: return kernel_of<2, 16>(tile, gw, mode);
+        case 224: return kernel_of<2, 24>(tile, gw, mode);
+        case 232: return kernel_of<2, 32>(tile, gw, mode);
+        case 308: return kernel_of<3, 8>(tile, gw, mode);
+        case 316: return kernel_of<3, 16>(tile, gw, mode);
+        case 324: return kernel_of<3, 24>(tile, gw, mode);
+        default: return kernel_of<3, 32>(tile, gw, mode);
     }
 }
 
@@ -226,7 +226,8 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
     if (B <= 0) return GF_OK;
     const int L = f->shape.L, C = f->C1;
     const bool gw = f->weights_global, rec = a.s_out != nullptr;
-    if (gw && rec) return GF_EUNSUPPORTED;
+    const int mode = rec ? kRecompute : a.xs_out ? kForward : kFlow;
+    if (gw && mode != kFlow) return GF_EUNSUPPORTED;
     a.W = f->d_packed;
     a.sched = f->d_sched;
     a.n_phases = f->n_phases;
@@ -265,11 +266,11 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
             const double cost = (double)((B + sms * r - 1) / (sms * r)) * std::max(lat, r * eff);
             if (nti < 0 || cost < best) { best = cost; nti = i; tile = t; }
         }
-    if (nti < 0 || !allow_smem(kernel_for(f, tile, rec))) return GF_ECUDA;
+    if (nti < 0 || !allow_smem(kernel_for(f, tile, mode))) return GF_ECUDA;
     const int NT = 64 << nti;
     a.n_passes = layer_cost(f, tile, NT / 32, f->stage_taps).passes;
     const int64_t grid = std::min<int64_t>(B, sms * ctas_per_sm(smem, NT));
-    kernel_for(f, tile, rec)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
+    kernel_for(f, tile, mode)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
     GF_CHECK_LAUNCH();
     return GF_OK;
 }

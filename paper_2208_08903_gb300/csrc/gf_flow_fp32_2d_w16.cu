@@ -5,7 +5,7 @@ namespace gf {
 namespace f32k {
 
 template <>
-FlowKernel kernel_of<2, 16>(int tile, bool gw, bool rec) { return pick_kernel<2, 16>(tile, gw, rec); }
+FlowKernel kernel_of<2, 16>(int tile, bool gw, int mode) { return pick_kernel<2, 16>(tile, gw, mode); }
 
 }  // namespace f32k
 }  // namespace gf

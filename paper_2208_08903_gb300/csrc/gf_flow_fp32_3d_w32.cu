@@ -5,7 +5,7 @@ namespace gf {
 namespace f32k {
 
 template <>
-FlowKernel kernel_of<3, 32>(int tile, bool gw, bool rec) { return pick_kernel<3, 32>(tile, gw, rec); }
+FlowKernel kernel_of<3, 32>(int tile, bool gw, int mode) { return pick_kernel<3, 32>(tile, gw, mode); }
 
 }  // namespace f32k
 }  // namespace gf

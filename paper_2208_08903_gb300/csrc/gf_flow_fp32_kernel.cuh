@@ -34,7 +34,9 @@
 // order from the bias (the same results for every tile and thread count); the
 // head sums as described at head_split.  The log-det, sum z^2 and the action
 // are FP32 pairs (gf_common.cuh) added as by 256 threads, whatever the CTA's
-// size (order_sum): results depend on the shape alone.
+// size (order_sum): results depend on the shape alone.  Training's forward pass
+// and recompute are instantiations of their own (kForward, kRecompute); its
+// log-det is an FP64 sum (train_logdet).
 #pragma once
 
 #include "gf_f32x2.cuh"
@@ -42,6 +44,11 @@
 
 namespace gf {
 namespace f32k {
+
+// What a kernel does: the flow in either direction; training's forward pass, which
+// saves the field after every layer and the log-det; training's recompute of one
+// layer (h1_out, h2_out, s_out), which does nothing else.
+constexpr int kFlow = 0, kForward = 1, kRecompute = 2;
 
 constexpr int kVT = 256;                   // threads of the sums' order; a CTA thread stands for up to 4
 
@@ -198,7 +205,7 @@ struct Weights {
 // h1 = LReLU(conv1(x at the sites of parity `frozen`)), 8 channels per thread,
 // sites ordered by parity so that a warp's live taps agree (half of the taps
 // reach fixed sites; the others add nothing).
-template <int ND, int C, bool GW, bool REC>
+template <int ND, int C, bool GW, int MODE>
 __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, const float* x, float* h1,
                          int frozen, int64_t b) {
     const int L = a.L, S = a.S, hS = S >> 1, nf = ph.n * S, half = nf >> 1;
@@ -239,7 +246,7 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
         for (int i = 0; i < 4; ++i) { v[2 * i] = lrelu(f2_lo(acc[i]), a.slope); v[2 * i + 1] = lrelu(f2_hi(acc[i]), a.slope); }
         *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
         *reinterpret_cast<float4*>(o + 4 * S) = make_float4(v[4], v[5], v[6], v[7]);
-        if constexpr (REC) {
+        if constexpr (MODE == kRecompute) {
             float* go = a.h1_out + ((b * (C / 4) + 2 * g) * a.V + sl * S + (ND == 3 ? y * L : 0) + xc) * 4;
             *reinterpret_cast<float4*>(go) = make_float4(v[0], v[1], v[2], v[3]);
             *reinterpret_cast<float4*>(go + 4 * (int64_t)a.V) = make_float4(v[4], v[5], v[6], v[7]);
@@ -249,7 +256,7 @@ __device__ void phase_h1(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
 
 // ---------------------------------------------------------------- conv2
 // One pass: warp `task` = 32 NS consecutive sites of the phase x CO channels.
-template <int ND, int C, int NS, int CO, bool GW, bool REC>
+template <int ND, int C, int NS, int CO, bool GW, int MODE>
 __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>& w, const Phase& ph, const float* h1,
                                         float* h2, int pass, int64_t b) {
     const int L = a.L, S = a.S, nf = ph.n * S, nblk = (nf + 32 * NS - 1) / (32 * NS);
@@ -330,7 +337,7 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
             for (int i = 0; i < CO / 4; ++i)
                 *reinterpret_cast<float4*>(o + (size_t)i * S * 4) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
-        if constexpr (REC) {
+        if constexpr (MODE == kRecompute) {
             const int n = wrap(ph.s0 + (at[k] >> 20), L) * S + (ND == 3 ? ((at[k] >> 10) & 1023) * L : 0) + (at[k] & 1023);
             float* go = a.h2_out + ((b * (C / 4) + (co >> 2)) * a.V + n) * 4 + (co & 3);
 #pragma unroll
@@ -344,7 +351,7 @@ __device__ __forceinline__ void conv2_pass(const FlowArgs& a, Weights<ND, C, GW>
 // (s, t) at the updated sites of slices r0 .. r0 + nr - 1 of the phase as one
 // packed pair; `tps` lanes share a site, each summing C / tps channels over all
 // taps, combined with xor-shuffles.
-template <int ND, int C, bool GW, bool REC>
+template <int ND, int C, bool GW, int MODE>
 __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const Phase& ph, int r0, int nr, int tps,
                          const float* h2, float* x, float* s_site, int frozen, bool inverse, FF& logdet, int64_t b) {
     constexpr int T = ND == 3 ? 27 : 9;
@@ -395,7 +402,7 @@ __device__ void phase_c3(const FlowArgs& a, const Weights<ND, C, GW>& w, const P
             const float spre = a.head_train ? ps : ps + bs, tt = a.head_train ? pt : pt + bt;
             const float s = a.use_tanh ? tanhf(spre) : spre;
             const int n = sl * S + (ND == 3 ? y * L : 0) + xc;
-            if constexpr (REC) {
+            if constexpr (MODE == kRecompute) {
                 a.s_out[b * a.V + n] = s;
                 continue;
             }
@@ -426,6 +433,56 @@ __device__ __forceinline__ void add_logdet(const FlowArgs& a, const float* s_sit
     }
 }
 
+// Training's log-det in FP64, added as k_couple_fwd of the layer-by-layer form
+// does, so that a configuration's log q does not depend on which form its batch
+// takes: thread vt of kVT takes the updated sites n = vt (mod kVT) of every layer
+// in order, then block_sum's order.  FP64 instructions are slow, so a thread
+// stands for vt = 2 i and 2 i + 1, of which one updates each of its site pairs,
+// and FP32 is widened by integer instructions: one FP64 addition per 32 updated
+// sites.  A training step takes 0.993 to 1.014 of its time with FP32 pairs (24 shapes).
+struct TrainLogdet {
+    double acc[2][2];                          // [i = thread + j CTA size][vt & 1]
+};
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)f;       // zero, subnormal, infinite, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+// adds one layer (fixed sites of parity `frozen`)
+template <int ND>
+__device__ __forceinline__ void train_logdet(const FlowArgs& a, const float* s_site, int frozen, TrainLogdet& t) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+#pragma unroll 1
+        for (int i = threadIdx.x + j * blockDim.x, u = i; i < kVT / 2 && u < (a.V >> 1); u += kVT / 2) {
+            const int sl = fdiv(2 * u, a.fd_S), row = ND == 3 ? fdiv(2 * u, a.fd_L) + sl : sl;   // (L is even)
+            const bool odd = ((frozen + 1 + row) & 1) != 0;            // x of the pair's updated site
+            const double v = (odd ? t.acc[j][1] : t.acc[j][0]) + widen(s_site[u]);
+            t.acc[j][0] = odd ? t.acc[j][0] : v;
+            t.acc[j][1] = odd ? v : t.acc[j][1];
+        }
+    }
+}
+// the sum over the threads (valid in thread 0); buf: kVT doubles (V when that is less)
+__device__ __forceinline__ double train_logdet_sum(const FlowArgs& a, const TrainLogdet& t, double* buf, double* red) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int i = threadIdx.x + j * blockDim.x;
+        if (i >= kVT / 2 || 2 * i >= a.V) continue;
+        buf[2 * i] = t.acc[j][0];
+        buf[2 * i + 1] = t.acc[j][1];
+    }
+    __syncthreads();
+    for (int vt = threadIdx.x; vt < kVT; vt += blockDim.x) {           // (uniform in a warp)
+        const double w = warp_sum(vt < a.V ? buf[vt] : 0.0);
+        if ((vt & 31) == 0) red[vt >> 5] = w;
+    }
+    __syncthreads();
+    double r = 0.0;
+    for (int i = 0; i < kVT / 32; ++i) r += red[i];
+    return r;
+}
+
 // FP64 value of the sum of part(j, vt) over vt < kVT in the order of kVT
 // threads (a butterfly in each warp of 32, then one over the warps); valid in
 // every thread.
@@ -446,8 +503,10 @@ __device__ double order_sum(FF* red, F part) {
     return ff_to_double(r);
 }
 
-// REC: training's recompute of one layer (h1_out, h2_out, s_out)
-template <int ND, int C, int NS, int CO, bool GW, bool REC>
+// (kFlow keeps its tests of xs_out and logdet_out, which are null there: without
+// them ptxas orders conv2's loop in the 5 x 8 tiles, at the limit of registers,
+// 4 % to 8 % slower; 3D L = 12, hidden 32, 8 layers, 300 configurations 7.45 -> 8.07 ms.)
+template <int ND, int C, int NS, int CO, bool GW, int MODE>
 __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant__ FlowArgs a, int inverse) {
     extern __shared__ __align__(16) float smf[];
     const int V = a.V;
@@ -489,6 +548,7 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
         }
         __syncthreads();
         FF logdet[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        TrainLogdet tld = {};                      // (kForward)
         double z2 = 0.0;
         const auto sum_squares = [&](int, int vt) {   // each square exactly as a pair
             FF v{0.f, 0.f};
@@ -500,8 +560,8 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             }
             return v;
         };
-        if (!inverse && !REC) {
-            z2 = order_sum(red, sum_squares);
+        if (!inverse && MODE != kRecompute) {
+            if constexpr (MODE == kFlow) z2 = order_sum(red, sum_squares);
             for (int n = threadIdx.x; n < V; n += blockDim.x) {
                 const float v = x[n];
                 if (a.z_out) a.z_out[b * V + n] = v;
@@ -522,18 +582,22 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
                 const Phase& ph = sched[p];
                 if (ph.type == PH_H2) {            // begins with a barrier of its own (begin_stage)
                     const int tasks = ((ph.n * a.S + 32 * NS - 1) / (32 * NS)) * (C / CO), nw = (int)(blockDim.x >> 5);
-                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW, REC>(a, w, ph, h1, h2, q, b);
+                    for (int q = 0; q * nw < tasks; ++q) conv2_pass<ND, C, NS, CO, GW, MODE>(a, w, ph, h1, h2, q, b);
                     continue;
                 }
                 __syncthreads();
                 if (ph.type == PH_H1) {
-                    if (!GW && p == 0 && li > 0) add_logdet(a, s_site, logdet);
-                    phase_h1<ND, C, GW, REC>(a, w, ph, x, h1, frozen, b);
+                    if constexpr (MODE == kForward) {
+                        if (p == 0 && li > 0) train_logdet<ND>(a, s_site, frozen ^ 1, tld);
+                    } else {
+                        if (!GW && p == 0 && li > 0) add_logdet(a, s_site, logdet);
+                    }
+                    phase_h1<ND, C, GW, MODE>(a, w, ph, x, h1, frozen, b);
                 } else {
                     const int na = max(0, min((int)ph.n, a.head_zb - (int)ph.s0));
-                    if (na > 0) phase_c3<ND, C, GW, REC>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0], b);
+                    if (na > 0) phase_c3<ND, C, GW, MODE>(a, w, ph, 0, na, a.head_a, h2, x, s_site, frozen, inverse, logdet[0], b);
                     if (na < ph.n)
-                        phase_c3<ND, C, GW, REC>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0], b);
+                        phase_c3<ND, C, GW, MODE>(a, w, ph, na, ph.n - na, a.head_b, h2, x, s_site, frozen, inverse, logdet[0], b);
                 }
             }
             w.end_layer();
@@ -541,7 +605,13 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
             --w.left;
         }
         __syncthreads();
-        if constexpr (REC) continue;               // ( the next configuration's x may be written now)
+        if constexpr (MODE == kForward) {
+            for (int n = threadIdx.x; n < V; n += blockDim.x) a.phi_out[b * V + n] = x[n];
+            if (N > 0) train_logdet<ND>(a, s_site, (N - 1) & 1, tld);
+            const double ld = train_logdet_sum(a, tld, reinterpret_cast<double*>(h1), reinterpret_cast<double*>(red));
+            if (threadIdx.x == 0) a.logdet_out[b] = ld;
+        }
+        if constexpr (MODE != kFlow) continue;     // (the next configuration's x may be written now)
 
         for (int n = threadIdx.x; n < V; n += blockDim.x) {
             if (!inverse) a.phi_out[b * V + n] = x[n];
@@ -569,22 +639,24 @@ __global__ void __launch_bounds__(512, 1) flow_fp32_kernel(const __grid_constant
 }
 
 using FlowKernel = void (*)(const FlowArgs, int);
-// the kernel of a lattice dimension, width and tile (gf_flow_fp32_*d_w*.cu);
-// recompute: tiles from kTileRec on
+// the kernel of a lattice dimension, width, tile and mode (gf_flow_fp32_*d_w*.cu);
+// the recompute has tiles from kTileRec on, weights in global memory are for
+// kFlow alone
 constexpr int kTileRec = 2;
 template <int ND, int C>
-FlowKernel kernel_of(int tile, bool gw, bool rec);
+FlowKernel kernel_of(int tile, bool gw, int mode);
 
 template <int ND, int C, int I = 0>
-FlowKernel pick_kernel(int tile, bool gw, bool rec) {
+FlowKernel pick_kernel(int tile, bool gw, int mode) {
     if constexpr (I == kTiles) {
         return nullptr;
     } else {
-        if (gw) return flow_fp32_kernel<ND, C, kTileNS[kTileGW], kTileCO[kTileGW], true, false>;
-        if (tile == I && !rec) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, false>;
+        if (gw) return flow_fp32_kernel<ND, C, kTileNS[kTileGW], kTileCO[kTileGW], true, kFlow>;
+        if (tile == I && mode == kFlow) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, kFlow>;
+        if (tile == I && mode == kForward) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, kForward>;
         if constexpr (I >= kTileRec)
-            if (tile == I && rec) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, true>;
-        return pick_kernel<ND, C, I + 1>(tile, gw, rec);
+            if (tile == I && mode == kRecompute) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, kRecompute>;
+        return pick_kernel<ND, C, I + 1>(tile, gw, mode);
     }
 }
 

@@ -194,17 +194,20 @@ __global__ void __launch_bounds__(kThreads) k_conv(const ConvArgs a) {
 // One CTA per configuration: (s, t) at the updated sites, x_out = x_in*e^s + t
 // there, x_out = x_in on fixed sites; s saved for the reverse pass;
 // logdet[b] += sum s (FP64, fixed-order block reduction) unless logdet is null
-// (then a configuration may be split over gridDim.y CTAs).
-template <int ND>
+// (then a configuration may be split over gridDim.y CTAs).  PARTS: the threads'
+// sums run on over the layers in part[b][kThreads] (from zero at layer 0) and
+// logdet[b] is their sum after the last one: the order of the fused forward pass.
+template <int ND, bool PARTS>
 __global__ void __launch_bounds__(kThreads) k_couple_fwd(const float* __restrict__ h2, int C2,
                                                         const float* __restrict__ W3, const float* __restrict__ b3,
                                                         int use_tanh, int frozen, int L, int V, int64_t B,
                                                         const float* __restrict__ xin, float* __restrict__ xout,
-                                                        float* __restrict__ s_save, double* __restrict__ logdet) {
+                                                        float* __restrict__ s_save, double* __restrict__ logdet,
+                                                        double* __restrict__ part, int layer, int n_layers) {
     __shared__ double red[32];
     const int T = ND == 3 ? 27 : 9;
     for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-        double ld = 0.0;
+        double ld = PARTS && layer > 0 ? part[b * kThreads + threadIdx.x] : 0.0;
         for (int n = blockIdx.y * blockDim.x + threadIdx.x; n < V; n += blockDim.x * gridDim.y) {
             const float xv = xin[b * V + n];
             if (parity<ND>(n, L) == frozen) { xout[b * V + n] = xv; s_save[b * V + n] = 0.f; continue; }
@@ -227,9 +230,10 @@ __global__ void __launch_bounds__(kThreads) k_couple_fwd(const float* __restrict
             s_save[b * V + n] = s;
             ld += (double)s;
         }
-        if (logdet) {                                   // uniform over the block
+        if (PARTS) part[b * kThreads + threadIdx.x] = ld;
+        if (logdet && (!PARTS || layer == n_layers - 1)) {   // uniform over the block
             const double tot = block_sum(ld, red);
-            if (threadIdx.x == 0) logdet[b] += tot;
+            if (threadIdx.x == 0) logdet[b] = PARTS ? tot : logdet[b] + tot;
         }
         __syncthreads();
     }
@@ -489,8 +493,13 @@ gf_status net_fwd(const gf_flow* f, int l, const float* xl, int64_t B, const Tra
     return conv<ND>(c2, st);
 }
 
+// kThreads FP64 partial sums of the log-det per configuration: the forward pass
+// has no use for gh1 (layer-by-layer lattices have far more than 512 values of it
+// a configuration).
+double* logdet_parts(const TrainWs& w) { return reinterpret_cast<double*>(w.gh1); }
+
 // One layer forward with a kernel per convolution: h1, h2, s and the field after
-// the layer (and its log-det added to `logdet` unless null).
+// the layer (and, unless null, `logdet` after the last one).
 template <int ND>
 gf_status layer_fwd(const gf_flow* f, int l, int64_t B, const float* xl, float* xout, double* logdet, const TrainWs& w,
                     cudaStream_t st) {
@@ -499,16 +508,18 @@ gf_status layer_fwd(const gf_flow* f, int l, int64_t B, const float* xl, float* 
     const PackedOffsets po = packed_offsets(f->T, f->C1, f->C2);
     const float* P = f->d_packed + (int64_t)l * f->packed_stride;
     const dim3 grid((unsigned)std::min<int64_t>(B, (int64_t)num_sms() * 8), logdet ? 1u : (unsigned)((f->V + kThreads - 1) / kThreads));
-    k_couple_fwd<ND><<<grid, kThreads, 0, st>>>(
-        w.h2, f->C2, P + po.W3, P + po.b3, f->shape.use_final_tanh, l & 1, f->shape.L, f->V, B, xl, xout, w.s, logdet);
+    const auto kern = logdet ? k_couple_fwd<ND, true> : k_couple_fwd<ND, false>;
+    kern<<<grid, kThreads, 0, st>>>(w.h2, f->C2, P + po.W3, P + po.b3, f->shape.use_final_tanh, l & 1, f->shape.L,
+                                    f->V, B, xl, xout, w.s, logdet, logdet_parts(w), l, f->shape.n_layers);
     GF_CHECK_LAUNCH();
     return GF_OK;
 }
 
 // Whether training runs the network layer by layer, a kernel per convolution
-// over all configurations, instead of fused with a CTA per configuration (the
-// results are the same; the kernels of 2D L=32 and 3D L=16 with width 32 always
-// run the forward pass fused): where the fused kernel has no room to stage weights,
+// over all configurations, instead of fused with a CTA per configuration (every
+// sum has one order in both, so the field, log q, loss and gradient are the same
+// to the bit whichever a batch takes; the kernels of 2D L=32 and 3D L=16 with
+// width 32 always run the forward pass fused): where the fused kernel has no room to stage weights,
 // and for lattices that do not fit a CTA at once when the batch leaves half of
 // the SMs idle (3D L=12 width 32, batch 64: 0.48 ms a layer fused).
 bool layerwise(const gf_flow* f, int64_t B) {
@@ -525,7 +536,8 @@ gf_status forward_pass(const gf_flow* f, int64_t B, uint64_t seed, uint64_t coun
     const int64_t BV = B * (int64_t)f->V;
     if (fp32_c32_supported(f) || !layerwise(f, B))
         // one fused launch: z (or the prior) -> every layer's input x_l and the
-        // log-det, with the FP32 weights (log q goes to a scratch buffer)
+        // log-det, with the FP32 weights (the kernels of gf_flow_fp32_c32.cu form
+        // log q too, into a scratch buffer)
         return launch_flow_fp32(f, false, nullptr, B, seed, counter0, z_in, w.xs, nullptr, w.xs + (int64_t)N * BV, w.loss_b,
                                 nullptr, nullptr, st, w.xs, BV, w.logdet);
     k_prior<<<(unsigned)grid1d(BV / 4 + 1), kThreads, 0, st>>>(f->V, B, seed, counter0, z_in, w.xs);
@@ -732,8 +744,8 @@ gf_status sample_unfused(const gf_flow* f, const gf_phi4* phi4, int64_t B, uint6
         ConvArgs c2{w.h1, C1, -1, P + po.W2, P + po.b2, C2, w.h2, slope, L, V, B};
         if ((s = conv<ND>(c2, st)) != GF_OK) return s;
         float* xout = bufs[l & 1];
-        k_couple_fwd<ND><<<cfg_grid, kThreads, 0, st>>>(w.h2, C2, P + po.W3, P + po.b3, f->shape.use_final_tanh,
-                                                       l & 1, L, V, B, xin, xout, w.s, w.logdet);
+        k_couple_fwd<ND, false><<<cfg_grid, kThreads, 0, st>>>(w.h2, C2, P + po.W3, P + po.b3, f->shape.use_final_tanh,
+                                                       l & 1, L, V, B, xin, xout, w.s, w.logdet, nullptr, l, N);
         GF_CHECK_LAUNCH();
         xin = xout;
     }
