@@ -68,7 +68,12 @@
 // their own, and four groups where one configuration fills the SM took, in us:
 // 2D L = 32, hidden 32, 24 layers, 8192 configurations 13436 -> 12892; 2D
 // L = 64, hidden 16, 16 layers, density of 1500 4604 -> 3853; 3D L = 12, hidden
-// 16, 16 layers, 999 configurations 2981 -> 2559.
+// 16, 16 layers, 999 configurations 2981 -> 2559.  Two configurations per CTA leave
+// 80 registers a thread: what only thread 0 needs lives in shared memory, counts
+// are 32 bits and the prior's z^2 is summed before the layers (2D hidden 32 spilled
+// 144 bytes of stores, now 12): the first case 12901 -> 12722, the second 3841 ->
+// 3727, 2D L = 16, hidden 32, 8 layers, 16,384 configurations 3805 -> 3728, 3D L = 8,
+// hidden 16 7794 -> 7342.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -96,7 +101,7 @@ constexpr int kTcM = 128;                 // rows per tile (TMEM lanes)
 constexpr int kTcOut = 96;                // output positions per tile (6 of every 8 rows)
 constexpr int kTcRings = 16;              // TMEM accumulators of all epilogue groups (at most)
 constexpr int kTcMaxTiles = 64;           // tiles per layer (one completion barrier each)
-constexpr long long kTcWaitLimit = 1ll << 22;
+constexpr int kTcWaitLimit = 1 << 22;
 constexpr int kSmemPerCTA = 232448;       // 227 KB opt-in maximum per CTA
 
 struct TcGeom {
@@ -144,12 +149,17 @@ __host__ __device__ inline int tc8_tap(int nd, int k, int kh) {
     return ta + kh;
 }
 
+// A count of which only zero and the last two bits matter: it stays in 32 bits
+// (and in a register) however long a launch runs.
+__device__ __forceinline__ int next_count(int n) { return n < 0x7ffffffc ? n + 1 : n - 3; }
+__device__ __forceinline__ int64_t next_count(int64_t n) { return n + 1; }
+
 // Bounded wait for completion number n (0-based) of an mbarrier (phase parity
 // n & 1; every waiter has seen completion n - 1 already, so the parity names
 // completion n).  False when the limit ran out (the CTA's abort flag is raised
 // and GF_ETIMEOUT recorded) or another thread already gave up.
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, int64_t n, volatile int* abort_flag, int32_t* status) {
-    long long spins = 0;
+    int spins = 0;
     while (!mbar_try_wait(bar, (uint32_t)(n & 1))) {
         ++spins;
         if ((spins & 63) == 0 && *abort_flag) return false;
@@ -163,8 +173,8 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, int64_t n, volatile int* 
 }
 // Bounded wait ignoring the abort flag (teardown: issued work must finish
 // before its shared memory or TMEM is released).
-__device__ __forceinline__ void tc_drain(uint64_t* bar, int64_t n) {
-    for (long long spins = 0; !mbar_try_wait(bar, (uint32_t)(n & 1)) && spins < kTcWaitLimit; ++spins) {}
+__device__ __forceinline__ void tc_drain(uint64_t* bar, int n) {
+    for (int spins = 0; !mbar_try_wait(bar, (uint32_t)(n & 1)) && spins < kTcWaitLimit; ++spins) {}
 }
 
 __device__ __forceinline__ uint4 pack_bf16x8(const float* v) {
@@ -476,9 +486,8 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
     const uint32_t a_ks = 2u * (uint32_t)npos;
     const int wf_floats = (int)(g.wf_bytes >> 2);
     const int64_t b0 = (int64_t)blockIdx.x * H + h, bstride = (int64_t)gridDim.x * H;
-    const int64_t n_cfg = a.B > b0 ? (a.B - 1 - b0) / bstride + 1 : 0;
-    const int64_t total_steps = n_cfg * a.n_layers;   // this half's layer applications
-    int64_t w2_issued = -1, w3_issued = -1, wf_issued = -1;   // thread 0: the last staged steps
+    double* z2_s = reinterpret_cast<double*>(red + 26);   // thread 0: the prior sample's sum of squares
+    int* issued = reinterpret_cast<int*>(red + 24);   // thread 0: the last staged steps (-1: none) of W2, W3 and the FP32 part
     // epilogue warps: group eg (warps 4 + 4 eg .. 7 + 4 eg) takes the tiles
     // t = eg (mod NG) through its own TMEM ring; warp w reads lane quarter w mod 4
     const int eg = warp >= 4 ? (warp - 4) >> 2 : -1, q = warp & 3;
@@ -489,11 +498,11 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
         mbar_expect_tx(bar, bytes);
         bulk_g2s(dst, a.Wl + (size_t)(INVERSE ? a.n_layers - 1 - li : li) * g.layer_bytes + off, bytes, bar);
     };
-    const auto stage_w2 = [&](int64_t step, int li) { stage(li, w2s, 0, g.w2_bytes, bar_w2); w2_issued = step; };
-    const auto stage_w3 = [&](int64_t step, int li) { stage(li, w3s, g.w2_bytes, g.w3_bytes, bar_w3); w3_issued = step; };
-    const auto stage_wf = [&](int64_t step, int li) {
+    const auto stage_w2 = [&](int step, int li) { stage(li, w2s, 0, g.w2_bytes, bar_w2); issued[0] = step; };
+    const auto stage_w3 = [&](int step, int li) { stage(li, w3s, g.w2_bytes, g.w3_bytes, bar_w3); issued[1] = step; };
+    const auto stage_wf = [&](int step, int li) {
         stage(li, wfs + (int)(step & 1) * wf_floats, g.w2_bytes + g.w3_bytes, g.wf_bytes, bar_wf + (step & 1));
-        wf_issued = step;
+        issued[2] = step;
     };
 
     // one allocation for the CTA (warp 0 of half 0); half h uses columns
@@ -532,6 +541,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
         mbar_init(bar_fin, NG);                // one commit per issuing thread
         mbar_init(bar_stall, 1);
         *abort_flag = 0;
+        issued[0] = issued[1] = issued[2] = -1;
         fence_mbar_init();
     }
     // positions past the padded lattice feed only dropped rows of the last
@@ -542,7 +552,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
-    if (tid == 0 && total_steps > 0) {
+    if (tid == 0 && b0 < a.B && a.n_layers > 0) {
         stage_w2(0, 0);
         stage_w3(0, 0);
         stage_wf(0, 0);
@@ -565,15 +575,19 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
     const int row = 32 * q + lane, roff = 6 * (row >> 3) + (row & 7);
     const bool rvalid = (row & 7) >= 1 && (row & 7) <= 6;
 
-    int64_t step = 0;
+    int step = 0;                             // layer applications so far
     // the next accumulator of this thread's ring (issuing thread r: ring r;
     // epilogue group g: ring g) and how often it has been filled before
     int i2 = 0, i3 = 0;
-    int64_t k2 = 0, k3 = 0;
+    // (the type by the time of either: 32 bits where registers are short or where it
+    // was faster, us: log q of 2400 3D L = 12, hidden 8, 5406 -> 5302; with 16 channels
+    // 64 bits, log q of 16,384 2D L = 16, 8 layers, 2592 -> 2427)
+    using Fills = std::conditional_t<H == 2 && (CP == 32 ? !INVERSE : CP == 8 && INVERSE), int, int64_t>;
+    Fills k2 = 0, k3 = 0;
     for (int64_t b = b0; b < a.B; b += bstride) {
         // prior sample (sampling) or the given field (inverting)
-        FF sumz2{0.f, 0.f};
         if (!INVERSE) {
+            FF sumz2{0.f, 0.f};
             if (a.z_in) {
                 for (int n = tid; n < V; n += kTcThreads) {
                     const float v = __ldg(a.z_in + b * V + n);
@@ -595,32 +609,35 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                     }
                 }
             }
-            half_sync();
+            const double z2 = half_sum(sumz2);     // (its barriers make x visible)
+            if (tid == 0) *z2_s = z2;
             if (a.z_out)
                 for (int n = tid; n < V; n += kTcThreads) a.z_out[b * V + n] = x[n];
         } else {
             for (int n = tid; n < V; n += kTcThreads) x[n] = __ldg(a.phi_in + b * V + n);
+            half_sync();
         }
-        half_sync();
 
         FF logdet{0.f, 0.f};
-        for (int li = 0; li < a.n_layers; ++li, ++step) {
+        for (int li = 0; li < a.n_layers; ++li, step = next_count(step)) {
             const int l = INVERSE ? a.n_layers - 1 - li : li, next_li = li + 1 == a.n_layers ? 0 : li + 1;
             const int frozen = l & 1;
             const float* wf = wfs + (int)(step & 1) * wf_floats;
 
             // ---- conv1 -> h1 (BF16, padded, with periodic images)
             if (tc_wait(bar_wf + (step & 1), step >> 1, abort_flag, a.status)) {
-                if (tid == 0 && step + 1 < total_steps) stage_wf(step + 1, next_li);
+                if (tid == 0 && (next_li > 0 || b + bstride < a.B)) stage_wf(next_count(step), next_li);
                 // Two sites per thread share the weight loads; 16 channels per item,
                 // all 32 where one configuration's 12 warps have registers for them.
                 // A round of pairs must stand for two of single sites, and in 2D pairs gain
                 // with 32 channels alone (single -> pairs, us: 3D L = 8, hidden 8, 3000
                 // configurations, rounds 2 -> 1, 1902 -> 1827; 3D L = 12, hidden 8, 458,
-                // rounds 5 -> 3, 985 -> 1024; 2D L = 24, hidden 16, 3000 1587 -> 1685).
+                // rounds 5 -> 3, 985 -> 1024; 2D L = 24, hidden 16, 3000 1587 -> 1685) or with
+                // 8 and one large configuration per CTA (150 of 2D, 24 layers: L = 48 377 ->
+                // 370, L = 64 613 -> 608).
                 constexpr int CH = CP < 16 || (H == 1 && NG == 2) ? CP : 16, NCB = CP / CH;
                 const int rounds1 = (V * NCB + kTcThreads - 1) / kTcThreads, rounds2 = (V / 2 * NCB + kTcThreads - 1) / kTcThreads;
-                const bool pairs = (ND == 3 || CP == 32) && 2 * rounds2 <= rounds1;
+                const bool pairs = (ND == 3 || CP == 32) ? 2 * rounds2 <= rounds1 : H == 1 && CP == 8 && rounds1 >= 6;
                 if (halo_pass) {
                     if constexpr (ND == 2 && CP >= 16)
                         tc_conv1<ND, CP, CP / 16, CH, false>(g, wf, x, frozen, a.slope, act, tid, kTcThreads);
@@ -668,7 +685,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                                                (uint32_t)(NKG * N2), (uint32_t)(2 * N2), idesc2);
                         mma_commit(full2 + warp * kTcRing + i2);
                         mma_commit(done2 + t);
-                        if (++i2 == nb2) { i2 = 0; ++k2; }
+                        if (++i2 == nb2) { i2 = 0; k2 = next_count(k2); }
                     }
                 }
                 __syncwarp();
@@ -738,7 +755,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                     }
                     fence_before_sync();
                     mbar_arrive(empty2 + eg * kTcRing + i2);
-                    if (++i2 == nb2) { i2 = 0; ++k2; }
+                    if (++i2 == nb2) { i2 = 0; k2 = next_count(k2); }
                     // h2 of tile t may overwrite h1 once tiles t .. t + r_lag are done (holding
                     // it back until after the next tile's arithmetic was 10 % to 20 % slower)
                     const int need = t + r_lag < nt ? t + r_lag : nt - 1;
@@ -762,7 +779,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
             if (*abort_flag) break;
             fence_after_sync();
             // every conv2 MMA of this layer has completed: the next layer's W2 may land
-            if (tid == 0 && step + 1 < total_steps) stage_w2(step + 1, next_li);
+            if (tid == 0 && (next_li > 0 || b + bstride < a.B)) stage_w2(next_count(step), next_li);
 
             // ---- periodic images of h2
             tc_halo<ND, CP>(g, act, tid, kTcThreads);
@@ -785,7 +802,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                             issue_tile<ND, CP>(p_first - 1 + kTcOut * t, P, PP, d3, a0, b3d, a_ks,
                                                (uint32_t)(NKG * 16), (uint32_t)(2 * 16), idesc3);
                         mma_commit(full3 + warp * kTcRing + i3);
-                        if (++i3 == nb3) { i3 = 0; ++k3; }
+                        if (++i3 == nb3) { i3 = 0; k3 = next_count(k3); }
                     }
                 }
                 __syncwarp();
@@ -801,7 +818,7 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
                     tmem_ld_wait();
                     fence_before_sync();
                     mbar_arrive(empty3 + eg * kTcRing + i3);
-                    if (++i3 == nb3) { i3 = 0; ++k3; }
+                    if (++i3 == nb3) { i3 = 0; k3 = next_count(k3); }
                     // columns 2 dx + j: j = 0 s, 1 t of tap dx at the row's own position
                     const float sl = __shfl_up_sync(0xffffffffu, v[0], 1, 8);
                     const float tl = __shfl_up_sync(0xffffffffu, v[1], 1, 8);
@@ -829,26 +846,32 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
             if (*abort_flag) break;
             fence_after_sync();
             // every conv3 MMA of this layer has completed: the next layer's W3 may land
-            if (tid == 0 && step + 1 < total_steps) stage_w3(step + 1, next_li);
+            if (tid == 0 && (next_li > 0 || b + bstride < a.B)) stage_w3(next_count(step), next_li);
         }
         if (*abort_flag) break;
 
+        const double ld = half_sum(logdet);
+        double z2 = 0.0;
         if (INVERSE) {
+            FF sumz2{0.f, 0.f};
             for (int n = tid; n < V; n += kTcThreads) {
                 const float v = x[n];
                 const float p = v * v;
                 ff_add(sumz2, FF{p, fmaf(v, v, -p)});
                 if (a.z_out) a.z_out[b * V + n] = v;
             }
+            z2 = half_sum(sumz2);
         } else {
             for (int n = tid; n < V; n += kTcThreads) a.phi_out[b * V + n] = x[n];
+            if (tid == 0) z2 = *z2_s;
         }
-        const double ld = half_sum(logdet);
-        const double z2 = half_sum(sumz2);
         double S = 0.0;
         if (!INVERSE && a.has_phi4) S = half_sum(action_part<ND>(x, L, V, a.c2d_ff, a.lam_ff, tid, kTcThreads));
         if (tid == 0) {
-            const double logr = -0.5 * z2 - 0.5 * (double)V * LOG_2PI;
+            // (the product that is fused, spelled out where the sampling kernels would
+            // differ in it; spelled out, the inverse ones take 2 % longer)
+            const double logr = INVERSE ? -0.5 * z2 - 0.5 * (double)V * LOG_2PI
+                                        : fma(-0.5, z2, -__dmul_rn(0.5 * (double)V, LOG_2PI));
             const double logq = logr - ld;
             a.logq_out[b] = logq;
             if (!INVERSE && a.has_phi4) {
@@ -862,9 +885,9 @@ __global__ void __launch_bounds__(tc_threads<NG>() * H, 1) flow_tc_kernel(const 
     // abort) finish before their shared memory and TMEM are released
     if (warp < NG && lane == 0) mma_commit(bar_fin);
     if (tid == 0) {
-        if (w2_issued >= 0) tc_drain(bar_w2, w2_issued);
-        if (w3_issued >= 0) tc_drain(bar_w3, w3_issued);
-        if (wf_issued >= 0) tc_drain(bar_wf + (wf_issued & 1), wf_issued >> 1);
+        if (issued[0] >= 0) tc_drain(bar_w2, issued[0]);
+        if (issued[1] >= 0) tc_drain(bar_w3, issued[1]);
+        if (issued[2] >= 0) tc_drain(bar_wf + (issued[2] & 1), issued[2] >> 1);
         tc_drain(bar_fin, 0);
     }
     fence_before_sync();
