@@ -204,14 +204,15 @@ __device__ __forceinline__ void pos_xyz(int p, int P, int PP, FastDiv fdP, FastD
     px = rem - py * P;
 }
 
-// LReLU of packed pairs: max(v, a v) for slopes a <= 1, the smaller of the two
-// above (the same numbers as v > 0 ? v : a v, in half the instructions).
+// LReLU of packed pairs: max(v, a v) for slopes 0 < a <= 1 (the same numbers as
+// v > 0 ? v : a v, in half the instructions; at a = 0 a v of -inf is NaN, which a
+// maximum would drop).
 template <int N>
 __device__ __forceinline__ void lrelu_pairs(const f32x2 (&v)[N], f32x2 slope2, float* out) {
     f32x2 av[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) av[i] = f2_mul(v[i], slope2);
-    if (f2_lo(slope2) <= 1.f) {
+    if (f2_lo(slope2) > 0.f && f2_lo(slope2) <= 1.f) {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             out[2 * i] = fmaxf(f2_lo(v[i]), f2_lo(av[i]));
@@ -220,8 +221,8 @@ __device__ __forceinline__ void lrelu_pairs(const f32x2 (&v)[N], f32x2 slope2, f
     } else {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            out[2 * i] = fminf(f2_lo(v[i]), f2_lo(av[i]));
-            out[2 * i + 1] = fminf(f2_hi(v[i]), f2_hi(av[i]));
+            out[2 * i] = f2_lo(v[i]) > 0.f ? f2_lo(v[i]) : f2_lo(av[i]);
+            out[2 * i + 1] = f2_hi(v[i]) > 0.f ? f2_hi(v[i]) : f2_hi(av[i]);
         }
     }
 }
