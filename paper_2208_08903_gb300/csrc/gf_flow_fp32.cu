@@ -3,8 +3,6 @@
 // size and conv2 tiles of a launch.
 #include <algorithm>
 #include <cstring>
-#include <mutex>
-#include <utility>
 
 #include "gf_flow_fp32_kernel.cuh"
 
@@ -133,21 +131,6 @@ int ctas_per_sm(size_t smem, int nt) {
     return std::min((int)(228 * 1024 / (smem + 1024)), 65536 / (128 * nt));
 }
 
-// Raises a kernel's shared-memory limit, once per device.
-bool allow_smem(FlowKernel kern) {
-    static std::mutex mu;
-    static std::vector<std::pair<int, FlowKernel>> done;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    std::lock_guard<std::mutex> lk(mu);
-    const std::pair<int, FlowKernel> key(dev, kern);
-    if (std::find(done.begin(), done.end(), key) != done.end()) return true;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget) != cudaSuccess)
-        return false;
-    done.push_back(key);
-    return true;
-}
-
 }  // namespace
 
 gf_status flow_fp32_configure(gf_flow* f) {
@@ -266,11 +249,16 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
             const double cost = (double)((B + sms * r - 1) / (sms * r)) * std::max(lat, r * eff);
             if (nti < 0 || cost < best) { best = cost; nti = i; tile = t; }
         }
-    if (nti < 0 || !allow_smem(kernel_for(f, tile, mode))) return GF_ECUDA;
+    if (nti < 0) return GF_ECUDA;
+    // (on every launch: a limit remembered from an earlier context does not hold
+    // after a device reset)
+    const FlowKernel kern = kernel_for(f, tile, mode);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBudget) != cudaSuccess)
+        return GF_ECUDA;
     const int NT = 64 << nti;
     a.n_passes = layer_cost(f, tile, NT / 32, f->stage_taps).passes;
     const int64_t grid = std::min<int64_t>(B, sms * ctas_per_sm(smem, NT));
-    kernel_for(f, tile, mode)<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
+    kern<<<(unsigned)grid, NT, smem, stream>>>(a, inverse ? 1 : 0);
     GF_CHECK_LAUNCH();
     return GF_OK;
 }
