@@ -176,7 +176,7 @@ gf_status flow_fp32_configure(gf_flow* f) {
                 if (L - a >= G) add(G);
                 else if (L - a > 2) add(L - a - 2);
             double c = 0;
-            for (int t = 0; t < kTiles; ++t) {
+            for (int t = tile_first(C); t < kTiles; ++t) {
                 const TileCost tc = layer_cost(f, t, 16, taps);
                 const double ct = std::max(tc.eff, tc.lat) + 12.0 * ((L + G - 1) / G + 1);   // phase overhead: barriers, tails
                 if (c == 0 || ct < c) c = ct;
@@ -240,7 +240,7 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
     int nti = -1, tile = 0;
     const int64_t sms = num_sms();
     double best = 0;
-    for (int t = gw ? kTileGW : rec ? kTileRec : 0; t < kTiles; ++t)
+    for (int t = gw ? kTileGW : rec ? kTileRec : tile_first(C); t < kTiles; ++t)
         for (int i = gw ? kCtaSizes - 2 : f->full ? 0 : kCtaSizes - 1; i < (gw ? kCtaSizes - 1 : kCtaSizes); ++i) {
             const int nt = 64 << i, r = (int)std::min<int64_t>((B + sms - 1) / sms, ctas_per_sm(smem, nt));
             const TileCost c = layer_cost(f, t, nt / 32, f->stage_taps);

@@ -93,6 +93,8 @@ constexpr int kTiles = kF32Tiles;
 constexpr int kTileNS[kTiles] = {1, 1, 2, 3, 5, 4};
 constexpr int kTileCO[kTiles] = {2, 4, 8, 8, 8, 8};
 constexpr int kTileGW = kTiles - 1;
+// Tiles of two channels are never the cheapest above width 8.
+constexpr int tile_first(int C) { return C > 8 ? 1 : 0; }
 
 __device__ __forceinline__ int wrap(int v, int L) { return v < 0 ? v + L : (v >= L ? v - L : v); }
 __device__ __forceinline__ float lrelu(float v, float a) { return v > 0.f ? v : a * v; }
@@ -650,6 +652,8 @@ template <int ND, int C, int I = 0>
 FlowKernel pick_kernel(int tile, bool gw, int mode) {
     if constexpr (I == kTiles) {
         return nullptr;
+    } else if constexpr (I < tile_first(C)) {
+        return pick_kernel<ND, C, I + 1>(tile, gw, mode);
     } else {
         if (gw) return flow_fp32_kernel<ND, C, kTileNS[kTileGW], kTileCO[kTileGW], true, kFlow>;
         if (tile == I && mode == kFlow) return flow_fp32_kernel<ND, C, kTileNS[I], kTileCO[I], false, kFlow>;
