@@ -132,8 +132,13 @@ __global__ void __launch_bounds__(kActThreads) action_kernel(int nd, int L, int 
 // field has a few sites far larger than the rest, sigma_H is large next to the
 // typical product and that is not enough: after the block sum, a
 // configuration whose estimated H error, 2^-45.5 sigma_H sqrt(V / 4), exceeds
-// 1e-13 max(|S|, 1) is summed again from global memory with a general pair
-// sum per site (site_term_ff, as the non-streaming kernel does).  That is slow,
+// 6e-14 max(|S|, 1) is summed again from global memory with a general pair
+// sum per site (site_term_ff, as the non-streaming kernel does).  (The limit:
+// over m2 = -6 .. -2, lam = 1 .. 10 the relative error of 400 actions is 5.8e-14
+// at most, median 1.5e-14; with 1e-13 it was 9.7e-14 and 1.6e-14, more than the
+// 6.4e-14 of folds of 8 sites, which had more configurations summed again.
+// Where a batch's configurations lie between the two limits it costs up to twice
+// the time, 54 -> 110 us for 16,384 of 2D L=32 at m2 = -4.9, lam = 2.3.)  That is slow,
 // so the folds are short: with a fold every 8 sites (sigma_H twice as large,
 // four times the error per fold) most configurations of a thermalised chain of
 // 3D L=16 (m2 = -6, lam = 5) were summed again: 418 us instead of 84 us for
@@ -306,10 +311,10 @@ __global__ void __launch_bounds__(kAsThreads) action_stream_kernel(int64_t B, co
             for (int w = 1; w < kAsWarps; ++w) ff_add(tot, pk[lane + 32 * w]);
             tot = warp_sum_ff(tot);
             // statistical size of the biased H error against the tolerance:
-            // 2^-45.5 sqrt(V/4) sigma_H <= 1e-13 max(|S|, 1), else (or NaN) the
+            // 2^-45.5 sqrt(V/4) sigma_H <= 6e-14 max(|S|, 1), else (or NaN) the
             // warp sums the configuration again from global memory, a general
             // pair sum per site
-            const float h_err = sH * (0.21022410f * sqrtf((float)(V / 4)));
+            const float h_err = sH * (0.35037350f * sqrtf((float)(V / 4)));
             if (!(h_err <= fmaxf(fabsf(tot.hi), 1.f))) {
                 const float* g = phi + b * V;
                 FF a{0.f, 0.f};
