@@ -234,7 +234,12 @@ gf_status launch_plan(const gf_flow* f, FlowArgs& a, bool inverse, cudaStream_t 
     const size_t smem = plan_smem(f, f->R, f->n_phases, gw, f->stage_taps, f->two_small, &a);
 
     // CTA size and tile: those that finish the batch soonest (estimated: conv2
-    // at its bound plus a fixed time per layer for the phases' latencies);
+    // at its bound plus a fixed time per layer for the phases' latencies; against
+    // every tile and CTA size on 50 lattices and widths at 64 to 4000 configurations
+    // the pick takes 1.00 of the best one's time at the median, 1.13 at the 90th
+    // percentile and 1.31 at worst, large batches of small lattices, which run best
+    // with 4 x 8 tiles and fewer threads: 3D L = 8, hidden 8, 4000 1575 against
+    // 1202 us);
     // 512 threads where the slices leave room for one CTA (256 with weights in
     // global memory, where the order of the sums is the CTA's own).
     int nti = -1, tile = 0;

@@ -24,8 +24,8 @@
 //
 // Measured against a kernel of 256 threads with scalar 4 x 8 tiles, weights read
 // from global memory and the phase headers fetched one by one: 3D L=12 width
-// 32, 16 couplings, batch 300: 42.7 -> 15.2 ms (32 TFLOP/s, FP32 pipe 49 %
-// active); 2D L=64 width 32: 20.4 -> 40.5 TFLOP/s; 2D L=8 width 8, 64
+// 32, 16 couplings, batch 300: 42.7 -> 14.8 ms (32 TFLOP/s; issue slots 50 %
+// active, the FMA pipe about 40 %); 2D L=64 width 32: 20.4 -> 40.5 TFLOP/s; 2D L=8 width 8, 64
 // configurations: 100 -> 59 us, 16,384: 4.2 -> 12.9 TFLOP/s.  One kernel per
 // tile: with the tile chosen inside one kernel the accumulators were spilled
 // around every weight stage (41 ms).
@@ -441,7 +441,7 @@ __device__ __forceinline__ void add_logdet(const FlowArgs& a, const float* s_sit
 // in order, then block_sum's order.  FP64 instructions are slow, so a thread
 // stands for vt = 2 i and 2 i + 1, of which one updates each of its site pairs,
 // and FP32 is widened by integer instructions: one FP64 addition per 32 updated
-// sites.  A training step takes 0.993 to 1.014 of its time with FP32 pairs (24 shapes).
+// sites.  A training step takes 0.986 to 1.007 of its time with FP32 pairs (24 shapes).
 struct TrainLogdet {
     double acc[2][2];                          // [i = thread + j CTA size][vt & 1]
 };

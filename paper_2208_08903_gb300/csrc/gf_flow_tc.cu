@@ -62,7 +62,7 @@
 // copies.
 //
 // What bounds it: chains of waits within a configuration, not the tensor pipe
-// (15 % busy).  2D L = 32, hidden 32, two configurations per CTA, cycles per
+// (20 % busy).  2D L = 32, hidden 32, two configurations per CTA, cycles per
 // layer: conv1 11 K, conv2 20 K, halo 0.5 K, head 8 K.  Packed FP32 pairs in
 // conv1 and the epilogue, conv1's images as predicated stores or a pass of
 // their own, and four groups where one configuration fills the SM took, in us:
@@ -239,9 +239,10 @@ __device__ __forceinline__ void load_pairs(f32x2 (&w)[N / 2], const float* p) {
 
 // conv1: h1 = LReLU(W1 * (x at the frozen sites) + b1) for every site, BF16, at
 // the site's padded position and its periodic images.  Sites are ordered
-// (parity, site), so a warp holds one site parity (V a multiple of 128) and the
-// live taps (those that reach frozen sites) are the same for the whole warp; the
-// weight loads are broadcasts.  A thread takes NS sites of one parity (j and
+// (parity, site), so that a warp holds one site parity and the live taps (those
+// that reach frozen sites) are the same for the whole warp (but for one warp where
+// V / (2 NS) is no multiple of 32, as in 3D L = 12: it issues both sets of taps);
+// the weight loads are broadcasts.  A thread takes NS sites of one parity (j and
 // j + V/(2 NS)) and CH of the channels, so each weight load feeds NS sites, as
 // packed FMAs over channel pairs.  Site j of parity q (rows y + L z in order, x
 // fastest in a row): x = 2 (j mod L/2) + ((q + y + z) mod 2).
@@ -437,7 +438,7 @@ __device__ __forceinline__ void issue_tile_c8(int first, int P, int PP, uint32_t
     }
 }
 
-// H halves of 12 warps each run one configuration at a time on their own
+// H halves of 4 + 4 NG warps each run one configuration at a time on their own
 // shared memory, TMEM columns and barriers (bar.sync 1 + half between
 // their phases), so that one half's CUDA-core phases overlap the other's
 // tensor-core phases: the runtime places a single CTA of a tcgen05 kernel

@@ -21,7 +21,10 @@
 // the stages don't fit beside them, the weights are read through L1.
 //
 // What bounds it: the latency of shared-memory loads and barriers with few warps
-// (registers, or the buffers' shared memory, allow 16 to 24 an SM).  One site per
+// (registers, or the buffers' shared memory, allow 16 to 24 an SM), and registers:
+// one kernel holds up to three forms of the hidden convolution and of the head, and
+// each of the six instantiations spills 1.2 to 1.9 KB of stores and 0.6 to 1.3 KB of
+// loads a thread at 80 or 128 registers (the former one-site kernel up to 32 bytes).  One site per
 // thread with the weights through L1 was bound by load issue (8 FMAs to 3 loads)
 // and waited for L2 at the start of every convolution: 2D L = 16, 12 layers,
 // widths 16, 16, 8, 5 taps, 500 configurations 3004 us, now 1319 (23 TFLOP/s);

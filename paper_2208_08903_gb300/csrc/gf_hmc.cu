@@ -18,7 +18,7 @@
 // serves, and exchanged by shuffles.  Measured, 20 steps, against the form with
 // the Laplacian, force and energies written out (18 FP64 instructions a step)
 // and four lanes evaluating every block: 512 chains of 3D L=16 2.39 -> 1.18 ms,
-// 152 chains 0.60 -> 0.30 ms, 400 chains of 2D L=64 1.58 -> 0.71 ms.  What is
+// 152 chains 0.60 -> 0.30 ms, 400 chains of 2D L=64 1.58 -> 0.73 ms.  What is
 // left above the instruction count is the SMs that hold 4 of the 512 chains
 // while others hold 3.
 #include <algorithm>
